@@ -88,7 +88,7 @@ cudaError_t commit_ordered(gem_ctx* h, const int* order, const float* const* gra
   a.pi_counts = pi_counts;
   a.pi_seg = pi_seg;
   a.pi_nseg = pi_nseg;
-  a.count_smem_at = 0;
+  a.lane_rows = 0;
   a.theta = h->theta;
   a.m = h->m;
   a.s = h->s;
@@ -123,21 +123,21 @@ cudaError_t commit_ordered(gem_ctx* h, const int* order, const float* const* gra
     a.K = kc;
     a.record_pi = 0;
     for (int k = 0; k < kc; ++k) {
-      a.pi_out[k] = pi_out ? pi_out[k0 + k] : nullptr;
-      if (a.pi_out[k]) a.record_pi = 1;
+      a.commit[k].pi_out = pi_out ? pi_out[k0 + k] : nullptr;
+      if (a.commit[k].pi_out) a.record_pi = 1;
     }
     for (int k = 0; k < kc; ++k) {
       const int w = order[k0 + k];
-      a.worker[k] = w;
-      a.grad[k] = grads[k0 + k];
+      a.commit[k].row = (long long)w * (long long)(h->stride * sizeof(float));
+      a.commit[k].grad = grads[k0 + k];
       // staleness: commits by the other workers since w's last commit (and pull)
       const int64_t tau = h->clock - h->last[size_t(w)] - 1;
       h->last[size_t(w)] = h->clock;
       h->clock += 1;
       // adaptive staleness: pi = 1 / (tau + 1) in fp32 (IEEE division); DOWNPOUR: pi = 1
-      a.pi[k] = h->mode == GEM_MODE_ADAPTIVE ? 1.0f / (static_cast<float>(tau) + 1.0f) : 1.0f;
+      a.commit[k].pi = h->mode == GEM_MODE_ADAPTIVE ? 1.0f / (static_cast<float>(tau) + 1.0f) : 1.0f;
     }
-    plan_slots(a);
+    plan_slots(a, order + k0);
     const cudaError_t e = launch_commit_batch(a, h->sm_count, h->stream);
     if (e != cudaSuccess) return e;
     h->launches += 1;

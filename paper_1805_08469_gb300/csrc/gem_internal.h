@@ -30,9 +30,45 @@ enum RuleKind : int {
   kRuleMomentum = 3,  // the proxy itself: theta += (m_w <- mu m_w + dtheta); no factor
 };
 
+// L2 policy of a store.
+enum L2Hint : uint8_t { kL2Normal = 0, kL2Keep = 1, kL2Stream = 2 };
+
+// How a commit of a launch reads and leaves its worker's m_w and s_w (one word, so that the
+// kernel reads it with one load).
+//   - slot_out >= 0 (rules with a moment): the worker commits again later in the launch and
+//     its lanes stay in that shared-memory slot instead of going to global memory; its next
+//     commit takes them from the slot of the same number, slot_in.
+//   - slot_in or slot_out < 0: from or to global memory.
+//   - keep_s (rules that do not read s_w): 0 skips the store of s_w when the worker commits
+//     again in the launch (nothing reads it before that).
+//   - l2: policy of the commit's stores of m_w and s_w to global memory (launches of more than
+//     kSmallBatch commits, rules with a moment): kL2Keep when a later commit of the launch
+//     reads them back from global memory, kL2Stream at the worker's last commit of the launch.
+struct CommitCtl {
+  uint32_t bits;
+  CommitCtl() = default;
+  __host__ __device__ CommitCtl(int in, int out, bool keep_s, int l2)
+      : bits(uint32_t(uint8_t(in)) | uint32_t(uint8_t(out)) << 8 | uint32_t(keep_s) << 16 | uint32_t(l2) << 24) {}
+  __host__ __device__ int slot_in() const { return int8_t(bits); }
+  __host__ __device__ int slot_out() const { return int8_t(bits >> 8); }
+  __host__ __device__ bool keep_s() const { return (bits >> 16 & 1u) != 0; }
+  __host__ __device__ int l2() const { return int(bits >> 24); }
+  __host__ __device__ void set_slot_in(int v) { bits = (bits & ~0xFFu) | uint8_t(v); }
+  __host__ __device__ void set_slot_out(int v) { bits = (bits & ~0xFF00u) | uint32_t(uint8_t(v)) << 8; }
+};
+
+// One commit of a launch (read by the kernel through one address).
+struct Commit {
+  const float* grad;     // its gradient, P floats
+  long long row;         // byte offset of its worker's row in m and s
+  float* pi_out;         // receives its scaling factors, P floats, or null
+  CommitCtl ctl;
+  float pi;              // kRuleFixed: its scaling factor
+};
+
 // Arguments of one launch of the fused commit kernel, for up to KCAP commits.  Launches of
-// at most kSmallBatch commits (single commits, the segments of the simulators) pass the
-// small form: the kernel parameters then take about 1 KB instead of 5.5 KB.
+// at most kSmallBatch commits (the segments of the simulators) and single commits pass a
+// shorter form: the kernel parameters then take about 1 KB or 100 bytes instead of 6.5 KB.
 template <int KCAP>
 struct BatchArgsT {
   float* theta;                            // [stride]
@@ -44,58 +80,37 @@ struct BatchArgsT {
   int K;                                   // commits in this launch, 1..KCAP
   int rule;                                // RuleKind
   float energy_scale;                      // kRuleScaled: factor on |m_w|
-  const float* grad[KCAP];                 // gradient of commit k, P floats
-  int worker[KCAP];                        // worker of commit k
-  float pi[KCAP];                          // kRuleFixed: scaling factor of commit k
-  int record_pi;                           // 1: pi_out[k] (when not null) receives pi
-  float* pi_out[KCAP];                     // scaling factors of commit k, P floats, or null
-  // Factor counts of a recording launch (null: none).  For every commit k with pi_out[k]
+  int record_pi;                           // 1: a commit's pi_out, when not null, receives its factors
+  Commit commit[KCAP];
+  // Factor counts of a recording launch (null: none).  For every commit k with pi_out
   // set and every segment s = [pi_seg[s], pi_seg[s + 1]) of the coordinates, the number of
   // recorded factors whose sign bit is set (below +0 in the total order of the medians) is
   // added to pi_counts[2 (k pi_nseg + s)] and the number equal to +0 to the word after it.
-  // The block keeps its counts in dynamic shared memory from float4 count_smem_at on.
   unsigned* pi_counts;
   const long long* pi_seg;                 // device array [pi_nseg + 1], non-decreasing
   int pi_nseg;
-  int count_smem_at;
-  // On-chip reuse of a worker that commits again later in the launch (energy rules):
-  // commit k keeps its m_w, s_w lanes in shared-memory slot slot_out[k] instead of writing
-  // them to global memory, and the worker's next commit reads them from slot_in[k];
-  // -1 means global memory.  Fixed-factor rules: keep_s[k] = 0 skips the store of s_w
-  // when the worker commits again in the launch (nothing reads it before that).
-  int8_t slot_in[KCAP];
-  int8_t slot_out[KCAP];
-  uint8_t keep_s[KCAP];
-  // L2 policy of commit k's stores of m_w and s_w to global memory (launches of more than
-  // kSmallBatch commits, energy rules): kL2Keep when a later commit of the launch reads
-  // them back from global memory (no slot), kL2Stream at the worker's last commit of the
-  // launch, kL2Normal otherwise.
-  uint8_t l2[KCAP];
+  int lane_rows;                           // dynamic shared memory: rows of a 16-byte lane per thread
 };
 using BatchArgs = BatchArgsT<kMaxBatchPerLaunch>;
-enum L2Hint : uint8_t { kL2Normal = 0, kL2Keep = 1, kL2Stream = 2 };
 constexpr int kSmallBatch = 32;
 
-// Shared-memory slots of the commit kernel (m_w and s_w lanes of one worker per slot), and
-// the shortest repeat distance (in commits) given a slot: shorter repeats are served by L2.
+// Shared-memory slots of the commit kernel (a worker's m_w and s_w lanes, 32 bytes per
+// thread and slot), and the commits whose copies a thread has in flight (rules with a moment):
+// 3 stages and 8 slots of a 128-thread block take 50 KB, four blocks per SM.  Measured at
+// P = 25M, n = 100 (us per 100 commits): 4 stages and 6 slots 5,170, 2 and 5 (six blocks)
+// 5,346, 4 and 12 (three blocks) 5,159, 2 and 9 5,737; at P = 1.2M, n = 20: 189, 191, 232, 208,
+// against 190.
 #ifndef GEM_COMMIT_SLOTS
-#define GEM_COMMIT_SLOTS 6
-#endif
-#ifndef GEM_COMMIT_SLOT_MIN_DISTANCE
-#define GEM_COMMIT_SLOT_MIN_DISTANCE 4
-#endif
-#ifndef GEM_COMMIT_REG_SLOTS
-#define GEM_COMMIT_REG_SLOTS 1
+#define GEM_COMMIT_SLOTS 8
 #endif
 constexpr int kCommitSlots = GEM_COMMIT_SLOTS;
-// Slots held in registers: ids kCommitSlots .. kCommitSlots + kRegSlots - 1 (one measured
-// best: a second pushes the kernel past 64 registers into a spill).
-constexpr int kRegSlots = GEM_COMMIT_REG_SLOTS;
-constexpr int kTotalSlots = kCommitSlots + kRegSlots;
-constexpr int kSlotMinDistance = GEM_COMMIT_SLOT_MIN_DISTANCE;
+#ifndef GEM_COMMIT_DEPTH
+#define GEM_COMMIT_DEPTH 3
+#endif
+constexpr int kCommitDepth = GEM_COMMIT_DEPTH;
 
-// Fill slot_in, slot_out, keep_s and l2 of a launch from its a.K workers.
-void plan_slots(BatchArgs& a);
+// Fill the ctl of a launch's commits from the workers of its a.K commits.
+void plan_slots(BatchArgs& a, const int* worker);
 
 // Launch the fused commit kernel for a.K commits on `stream`.
 cudaError_t launch_commit_batch(const BatchArgs& a, int sm_count, cudaStream_t stream);
