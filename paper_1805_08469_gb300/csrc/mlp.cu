@@ -19,6 +19,7 @@
 // Precision.  Every product runs in one grouped SIMT GEMM kernel that reads either operand
 // layout; with GEM_MLP_TF32 it rounds each operand to TF32 as it loads it (products of TF32
 // values are exact in fp32; the sums stay fp32).
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include <cstdint>
@@ -65,6 +66,10 @@ struct Operand {
   long long group_stride;  // elements between the operands of consecutive groups
   long long ld;            // leading dimension of its row-major storage
   int by_worker;           // group g uses index workers[g] (GEM state) instead of g (scratch)
+  // CUDA-core path only: storage row r of group g is row rows[g * rows_per_group + r] of base
+  // (minibatch rows read in place from the data set); null: row r of group g's operand
+  const int32_t* rows;
+  int rows_per_group;
 };
 
 struct GemmArgs {
@@ -77,12 +82,14 @@ struct GemmArgs {
   long long bias_group_stride;
   const float* mask;  // by group, keep C(m, n) where mask(m, n) > 0
   long long mask_group_stride, ldmask;
-  // split-K: blockIdx.z = group * ksplit + split; split s sums k in [s kchunk, (s+1) kchunk)
-  // and writes its raw partial sums to ws + (group * ksplit + s) * M * N (row-major, ld N)
+  // split-K: blockIdx.z = group * ksplit + split; split s sums k in [s kchunk, (s+1) kchunk).
+  // Tensor cores: it writes its raw partial sums to ws + (group * ksplit + s) * M * N
+  // (row-major, ld N).  CUDA cores: the splits of a tile are a cluster and add them on chip.
   int ksplit;
   int kchunk;
   float* ws;            // null: no split
   long long ws_floats;  // capacity of ws
+  int can_split;        // CUDA-core path: K may be cut
   // tensor-core path: floats addressable from each operand's base (0: unknown, which keeps
   // the product off that path) and the error word its kernels report to
   long long a_extent, b_extent, c_extent, bias_extent, mask_extent;
@@ -102,6 +109,27 @@ __device__ __forceinline__ float to_tf32(float x) {
   uint32_t u = __float_as_uint(x);
   if ((u & 0x7F800000u) != 0x7F800000u) u = (u + 0x1000u) & 0xFFFFE000u;
   return __uint_as_float(u);
+}
+
+// ---- asynchronous copies
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src, int src_bytes) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gmem_src), "r"(src_bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src, int src_bytes) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(gmem_src), "r"(src_bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ uint32_t tf32_bits(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return r;
 }
 
 // Four consecutive elements (outer, inner .. inner + 3) of a row-major view with leading
@@ -131,7 +159,8 @@ __device__ __forceinline__ float4 stage_quad(const float* base, long long ld, bo
   return v;
 }
 
-// C[g] (M x N) = epilogue( op(A[g]) op(B[g]) ).  A_KMAJOR: A(m, k) at A[m*lda + k], else at
+// C[g] (M x N) = epilogue( op(A[g]) op(B[g]) ), where there is enough work to be bound by the
+// FMAs (see small_product).  A_KMAJOR: A(m, k) at A[m*lda + k], else at
 // A[k*lda + m].  B_KMAJOR: B(k, n) at B[n*ldb + k], else at B[k*ldb + n].
 //
 // TBM x 64 tile per block of 2 TBM threads; thread (tx, ty) = (tid % 16, tid / 16) owns
@@ -274,6 +303,218 @@ gemm_grouped_kernel(const __grid_constant__ GemmArgs p) {
       C[m * p.ldc + n] = v;
     }
   }
+}
+
+// The same where latency bounds the product.  A_KMAJOR: A(m, k) at
+// A[m*lda + k], else at A[k*lda + m].  B_KMAJOR: B(k, n) at B[n*ldb + k], else at B[k*ldb + n].
+//
+// A block of 128 threads computes a BM x 64 tile, TM x TN outputs per thread (8 x 4 for BM =
+// 64, 4 x 4 for 32), each summed over k in order.  The k-tiles come through a
+// ring of kSimtStages stages of asynchronous copies, zero-filled at the edges: a K-major
+// operand lies [row][k] with a pitch of 20 floats, the other [k][row], and in both a
+// thread reads 16 bytes at a time without bank conflicts (rows of a K-major operand are dealt
+// to the threads in turn, of the other in runs of four), TM + TN reads per 4 TM TN FMAs.
+// K may be cut: the ksplit splits of a tile are one cluster, each leaves its partial tile in its
+// shared memory, and each adds a share of the rows over the splits, in order, applies the
+// epilogue and stores it: one launch, no workspace.  The sums are those of gemm_grouped_kernel
+// with splitk_reduce_kernel, in the same order, so the two give the same bits.
+constexpr int kSimtThreads = 128, kSimtStages = 4;
+
+template <int BM>
+struct SimtTile {
+  static constexpr int TM = BM == 32 ? 4 : 8, TN = 4;
+  static constexpr int TX = BN / TN, TY = BM / TM;   // threads along n and m
+  static_assert(TX * TY == kSimtThreads, "one thread per TM x TN outputs");
+};
+constexpr int kSimtPitch = BK + 4;   // floats between the rows of a K-major tile
+constexpr int kPartPitch = BN + 8;   // floats between the rows of a partial tile
+__host__ __device__ constexpr int simt_tile_floats(int rows, bool kmajor) {
+  return kmajor ? rows * kSimtPitch : BK * rows;
+}
+// dynamic shared memory in floats: the ring, or the partial tile that takes its place
+__host__ __device__ constexpr int simt_smem_floats(int bm, bool ak, bool bk) {
+  const int ring = kSimtStages * (simt_tile_floats(bm, ak) + simt_tile_floats(BN, bk));
+  const int part = bm * kPartPitch;
+  return ring > part ? ring : part;
+}
+
+// Issue the copies of k-tile [k0, k0 + 16) of an operand tile of R rows from row0 on into
+// dst.  src: the group's operand; idx (shared memory, or null): storage rows to read instead;
+// vec: its rows start on 16-byte boundaries.  Elements at rows >= rows_end or k >= k_end are
+// zeros.
+template <int R, bool KMAJOR>
+__device__ __forceinline__ void simt_stage(float* dst, const float* src, long long ld, const int32_t* idx,
+                                           bool vec, int row0, int rows_end, int k0, int k_end) {
+  constexpr int kQuads = R * BK / 4;
+#pragma unroll
+  for (int q0 = 0; q0 < kQuads; q0 += kSimtThreads) {
+    const int q = q0 + threadIdx.x;
+    if (kQuads % kSimtThreads != 0 && q >= kQuads) break;
+    int outer, inner, outer_end, inner_end;   // storage row and column of the quad
+    float* d;
+    if (KMAJOR) {
+      const int row = q / (BK / 4), k = q % (BK / 4) * 4;
+      d = dst + row * kSimtPitch + k;
+      outer = row0 + row;
+      inner = k0 + k;
+      outer_end = rows_end;
+      inner_end = k_end;
+    } else {
+      const int k = q / (R / 4), row = q % (R / 4) * 4;
+      d = dst + k * R + row;
+      outer = k0 + k;
+      inner = row0 + row;
+      outer_end = k_end;
+      inner_end = rows_end;
+    }
+    const int valid = outer < outer_end ? min(4, max(0, inner_end - inner)) : 0;
+    const long long r = valid > 0 && idx ? (long long)idx[outer] : (long long)outer;
+    const float* g = valid > 0 ? src + r * ld + inner : src;
+    if (vec) {
+      cp_async16(d, g, valid * 4);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) cp_async4(d + e, e < valid ? g + e : src, e < valid ? 4 : 0);
+    }
+  }
+}
+
+template <int BM, bool A_KMAJOR, bool B_KMAJOR, int EPI, bool TF32>
+__global__ void __launch_bounds__(kSimtThreads, 4)
+gemm_simt_kernel(const __grid_constant__ GemmArgs p) {
+  gem::pdl_entry();
+  using Tile = SimtTile<BM>;
+  constexpr int TM = Tile::TM, TN = Tile::TN, TX = Tile::TX, TY = Tile::TY;
+  constexpr int kA = simt_tile_floats(BM, A_KMAJOR), kStage = kA + simt_tile_floats(BN, B_KMAJOR);
+  extern __shared__ __align__(16) float simt_smem[];
+  __shared__ int32_t row_idx[kMaxBatch];
+  const int split = p.ksplit;
+  const int g = blockIdx.z / split, sk = blockIdx.z - g * split;
+  const int kbeg = sk * p.kchunk, kend = min(p.K, kbeg + p.kchunk);
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const float* A = p.A.base + (p.A.by_worker ? (long long)p.workers[g] : (long long)g) * p.A.group_stride;
+  const float* B = p.B.base + (p.B.by_worker ? (long long)p.workers[g] : (long long)g) * p.B.group_stride;
+  const int M = p.M, N = p.N;
+  const bool a_vec = (reinterpret_cast<uintptr_t>(A) & 15u) == 0 && (p.A.ld & 3) == 0;
+  const bool b_vec = (reinterpret_cast<uintptr_t>(B) & 15u) == 0 && (p.B.ld & 3) == 0;
+  const int32_t* idx = p.A.rows ? p.A.rows : p.B.rows;   // at most one operand reads by index
+  if (idx) {
+    const int n_rows = p.A.rows ? p.A.rows_per_group : p.B.rows_per_group;
+    for (int i = tid; i < n_rows; i += kSimtThreads) row_idx[i] = idx[(long long)g * n_rows + i];
+    __syncthreads();
+  }
+  const int32_t* a_idx = p.A.rows ? row_idx : nullptr;
+  const int32_t* b_idx = p.B.rows ? row_idx : nullptr;
+
+  const int nkt = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+  auto issue = [&](int kt) {
+    if (kt < nkt) {
+      float* st = simt_smem + kt % kSimtStages * kStage;
+      const int k0 = kbeg + kt * BK;
+      simt_stage<BM, A_KMAJOR>(st, A, p.A.ld, a_idx, a_vec, m0, M, k0, kend);
+      simt_stage<BN, B_KMAJOR>(st + kA, B, p.B.ld, b_idx, b_vec, n0, N, k0, kend);
+    }
+    cp_async_commit();
+  };
+  float acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+#pragma unroll
+  for (int kt = 0; kt < kSimtStages - 1; ++kt) issue(kt);
+
+  auto round = [](float v) { return TF32 ? __uint_as_float(tf32_bits(v)) : v; };
+#pragma unroll 1
+  for (int kt = 0; kt < nkt; ++kt) {
+    cp_async_wait<kSimtStages - 2>();
+    __syncthreads();   // everyone's copies of k-tile kt have landed; k-tile kt - 1 has been read
+    issue(kt + kSimtStages - 1);
+    const float* As = simt_smem + kt % kSimtStages * kStage;
+    const float* Bs = As + kA;
+#pragma unroll
+    for (int k = 0; k < BK; k += 4) {
+      float a[TM][4], b[TN][4];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        // K-major: row ty + TY i, k .. k + 3; else rows 4 ty .. 4 ty + 3 (+ 4 TY per four) at k + i % 4
+        const float4 v = *reinterpret_cast<const float4*>(
+            A_KMAJOR ? As + (ty + TY * i) * kSimtPitch + k : As + (k + i % 4) * BM + (i / 4) * (4 * TY) + 4 * ty);
+        const float e[4] = {round(v.x), round(v.y), round(v.z), round(v.w)};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (A_KMAJOR) a[i][q] = e[q];
+          else a[i / 4 * 4 + q][i % 4] = e[q];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const float4 v = *reinterpret_cast<const float4*>(
+            B_KMAJOR ? Bs + (tx + TX * j) * kSimtPitch + k : Bs + (k + j % 4) * BN + (j / 4) * (4 * TX) + 4 * tx);
+        const float e[4] = {round(v.x), round(v.y), round(v.z), round(v.w)};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (B_KMAJOR) b[j][q] = e[q];
+          else b[j / 4 * 4 + q][j % 4] = e[q];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i][q], b[j][q], acc[i][j]);
+    }
+  }
+
+  // tile coordinates of this thread's outputs
+  auto row_of = [&](int i) { return A_KMAJOR ? ty + TY * i : (i / 4) * (4 * TY) + 4 * ty + i % 4; };
+  auto col_of = [&](int j) { return B_KMAJOR ? tx + TX * j : (j / 4) * (4 * TX) + 4 * tx + j % 4; };
+  float* C = p.C + (long long)g * p.c_group_stride;
+  const float* bias = (EPI == kBias || EPI == kBiasRelu)
+                          ? p.bias + (long long)p.workers[g] * p.bias_group_stride : nullptr;
+  const float* mask = EPI == kMask ? p.mask + (long long)g * p.mask_group_stride : nullptr;
+  auto finish = [&](float v, int m, int n) {
+    if (EPI == kBias) v = v + bias[n];
+    if (EPI == kBiasRelu) v = fmaxf(v + bias[n], 0.f);
+    if (EPI == kMask) v = mask[m * p.ldmask + n] > 0.f ? v : 0.f;
+    C[m * p.ldc + n] = v;
+  };
+  if (split == 1) {
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int m = m0 + row_of(i);
+      if (m >= M) continue;
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int n = n0 + col_of(j);
+        if (n < N) finish(acc[i][j], m, n);
+      }
+    }
+    return;
+  }
+  // the cluster adds its partial tiles
+  cp_async_wait<0>();
+  __syncthreads();   // the ring's last k-tile has been read
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) simt_smem[row_of(i) * kPartPitch + col_of(j)] = acc[i][j];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();
+  const int rows = min(BM, M - m0), per = (rows + split - 1) / split;
+  const int r_end = min(rows, (sk + 1) * per);
+  const int c = tid % BN, n = n0 + c;
+  if (n < N) {
+    for (int r = sk * per + tid / BN; r < r_end; r += kSimtThreads / BN) {
+      float v = 0.f;
+      for (int q = 0; q < split; ++q) v += cluster.map_shared_rank(simt_smem, q)[r * kPartPitch + c];
+      finish(v, m0 + r, n);
+    }
+  }
+  cluster.sync();   // every partial tile has been read
 }
 
 // The same products with TF32 operands on the tensor cores (warp-level mma.sync, m16n8k8,
@@ -462,21 +703,6 @@ static_assert(kPipeBK % 8 == 0 && (64 * kPipeBK / 4) % 256 == 0, "k-tile must sp
 __host__ __device__ constexpr int pipe_tile_floats(int rows, bool kmajor) {
   return kmajor ? rows * (kPipeBK + 4) : kPipeBK * (rows + 8);
 }
-
-__device__ __forceinline__ uint32_t tf32_bits(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src, int src_bytes) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gmem_src), "r"(src_bytes)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Stage the k-tile [k0, k0 + 32) of an operand tile of R rows (m or n) starting at row0:
 // element (row, k) is at src[row * ld + k] (K-major) or src[k * ld + row].  Rows >= rows_end
@@ -1006,13 +1232,107 @@ bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
   }
 }
 
-template <int TBM, bool AK, bool BK_, int EPI>
-void launch_tile(const GemmArgs& a, int groups, bool tf32, cudaStream_t st) {
+// Whether latency, not the FMAs, bounds a CUDA-core product: below 40 million FMAs (about 0.5
+// us of every SM) a block has a handful of k-tiles, and waiting for each of them costs more
+// than multiplying it.  Measured, whole runs with gemm_grouped_kernel for every product and with
+// gemm_simt_kernel for every product: 784-64-10, n = 4 (1.6 to 6.4M FMAs per product) 1,018 and
+// 890 us; the MNIST network, n = 100 (3 to 50M) 1,130 and 1,092 us; 784-1000-1000-10, n = 30 in
+// fp32 (100M to 1.5G) 2,240 and 2,410 us; six gradients of 784-235-629-10, b = 74 (66 to 82M)
+// 140 and 148 us.
+bool small_product(int M, int N, int K, int groups) {
+  return (long long)M * N * K * groups < 40000000ll;
+}
+
+// How many parts a product's K is cut in on the CUDA cores: up to kMaxSplit while the product
+// has too few tiles to fill the GPU.  It decides the order of the sums, so it depends on the
+// product alone and not on the kernel that runs it.
+int simt_split(int M, int N, int K, int groups, bool can_split) {
+  const long long nt = (N + BN - 1) / BN;
+  int split = 1;
+  if (can_split && M <= 128 && nt * ((M + 127) / 128) * groups < GEM_SIMT_BIG_TILE_BLOCKS * kSmCountHint)
+    while (split < kMaxSplit && nt * ((M + 63) / 64) * groups * split < 4 * kSmCountHint &&
+           K / (2 * split) >= GEM_SIMT_MIN_CHUNK)
+      split *= 2;
+  return split;
+}
+
+template <int BM, bool AK, bool BK_, int EPI, bool TF32>
+cudaError_t launch_simt_tile(const GemmArgs& a, int groups, cudaStream_t st) {
+  constexpr int bytes = 4 * simt_smem_floats(BM, AK, BK_);
+  if (bytes > 40 * 1024) {   // with the row indices beyond the default limit
+    static bool configured[64] = {};   // one attribute call per instantiation and device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !configured[dev]) {
+      const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, AK, BK_, EPI, TF32>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+      if (e != cudaSuccess) return e;
+      if (dev >= 0 && dev < 64) configured[dev] = true;
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned((a.N + BN - 1) / BN), unsigned((a.M + BM - 1) / BM), unsigned(groups * a.ksplit));
+  cfg.blockDim = dim3(kSimtThreads);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;   // the splits of a tile
+  attr[1].val.clusterDim.x = 1;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = unsigned(a.ksplit);
+  cfg.attrs = attr;
+  cfg.numAttrs = a.ksplit > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, gemm_simt_kernel<BM, AK, BK_, EPI, TF32>, a);
+}
+
+// Rows per tile: 64, or 32 where 64 would leave half of the tile empty or SMs without a block.
+template <bool AK, bool BK_, int EPI, bool TF32>
+cudaError_t launch_simt(const GemmArgs& a, int groups, cudaStream_t st) {
+  const long long tiles64 = (long long)((a.M + 63) / 64) * ((a.N + BN - 1) / BN) * groups * a.ksplit;
+  if (a.M <= 32 || tiles64 < 2 * kSmCountHint) return launch_simt_tile<32, AK, BK_, EPI, TF32>(a, groups, st);
+  return launch_simt_tile<64, AK, BK_, EPI, TF32>(a, groups, st);
+}
+
+template <int TBM, bool AK, bool BK_, int EPI, bool TF32>
+void launch_tile(const GemmArgs& a, int groups, cudaStream_t st) {
   dim3 grid((a.N + BN - 1) / BN, (a.M + TBM - 1) / TBM, groups);
-  if (tf32)
-    gem::launch_pdl(gemm_grouped_kernel<TBM, AK, BK_, EPI, true>, grid, 2 * TBM, 0, st, a);
+  gem::launch_pdl(gemm_grouped_kernel<TBM, AK, BK_, EPI, TF32>, grid, 2 * TBM, 0, st, a);
+}
+
+// Adds the split-K partials of a product in its workspace.
+template <int EPI>
+void launch_reduce(const GemmArgs& a, int groups, cudaStream_t st) {
+  // float4 columns when every row of every array starts on a 16-byte boundary
+  auto al = [](const void* ptr, long long stride) {
+    return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0 && stride % 4 == 0;
+  };
+  const bool vec = a.N % 4 == 0 && al(a.C, a.c_group_stride) && a.ldc % 4 == 0 &&
+                   (!(EPI == kBias || EPI == kBiasRelu) || al(a.bias, a.bias_group_stride)) &&
+                   (EPI != kMask || (al(a.mask, a.mask_group_stride) && a.ldmask % 4 == 0));
+  const int V = vec ? 4 : 1;
+  dim3 grid(unsigned((a.N + 256 * V - 1) / (256 * V)), unsigned(a.M * groups));
+  if (vec)
+    gem::launch_pdl(splitk_reduce_kernel<EPI, 4>, grid, 256, 0, st, a);
   else
-    gem::launch_pdl(gemm_grouped_kernel<TBM, AK, BK_, EPI, false>, grid, 2 * TBM, 0, st, a);
+    gem::launch_pdl(splitk_reduce_kernel<EPI, 1>, grid, 256, 0, st, a);
+}
+
+// A product on the CUDA cores.
+template <bool AK, bool BK_, int EPI, bool TF32>
+cudaError_t launch_cuda_cores(GemmArgs a, int groups, cudaStream_t st) {
+  a.ksplit = simt_split(a.M, a.N, a.K, groups, a.can_split != 0);
+  a.kchunk = a.ksplit > 1 ? ((a.K + a.ksplit - 1) / a.ksplit + BK - 1) / BK * BK : a.K;
+  if (small_product(a.M, a.N, a.K, groups)) return launch_simt<AK, BK_, EPI, TF32>(a, groups, st);
+  const long long big = (long long)((a.N + BN - 1) / BN) * ((a.M + 127) / 128) * groups;
+  if (big >= GEM_SIMT_BIG_TILE_BLOCKS * kSmCountHint) {
+    launch_tile<128, AK, BK_, EPI, TF32>(a, groups, st);
+  } else {
+    launch_tile<64, AK, BK_, EPI, TF32>(a, groups * a.ksplit, st);
+    if (a.ksplit > 1) launch_reduce<EPI>(a, groups, st);
+  }
+  return cudaGetLastError();
 }
 
 bool operand_16b(const Operand& o) {
@@ -1040,11 +1360,10 @@ void launch_mma(const GemmArgs& a, int groups, cudaStream_t st) {
   }
 }
 
-// TF32 products run on the tensor cores (mma.sync), fp32 products on the CUDA cores.  The
-// large tile (128 x 128 on the tensor cores, 128 x 64 on the CUDA cores) when the launch
-// fills the GPU with at least two blocks per SM; otherwise the half-size tile and, when a
-// split-K workspace is given and K is long, up to kMaxSplit splits of K whose partial sums a
-// second kernel adds in a fixed order.
+// fp32 products run on the CUDA cores, TF32 products on the tensor cores (tcgen05 where its
+// kernel takes the product, else mma.sync).  On mma.sync: the 128 x 128 tile when the launch fills the GPU;
+// otherwise the half-size tile and, when a split-K workspace is given and K is long, up to
+// kMaxSplit splits of K whose partial sums a second kernel adds in a fixed order.
 template <bool AK, bool BK_, int EPI>
 cudaError_t launch_gemm(const GemmArgs& a_in, int groups, bool tf32, cudaStream_t st,
                         bool* on_tc = nullptr) {
@@ -1056,7 +1375,10 @@ cudaError_t launch_gemm(const GemmArgs& a_in, int groups, bool tf32, cudaStream_
   // gradients) would leave a 128-row tensor-core tile mostly empty or its pipeline idle:
   // they run on the CUDA cores, with the same TF32 operand rounding.
   const bool tc = tf32 && a.M >= 32 && a.K >= 32;
-  if (tc && a.a_extent > 0 && a.b_extent > 0 && a.c_extent > 0) {
+  if (!tc)
+    return tf32 ? launch_cuda_cores<AK, BK_, EPI, true>(a, groups, st)
+                : launch_cuda_cores<AK, BK_, EPI, false>(a, groups, st);
+  if (a.a_extent > 0 && a.b_extent > 0 && a.c_extent > 0) {
     // the 5th-generation tensor cores (tcgen05, accumulator in tensor memory), for products
     // whose layout, epilogue and alignment its kernel takes; the others stay on mma.sync
     gem::tc::Args t;
@@ -1090,45 +1412,23 @@ cudaError_t launch_gemm(const GemmArgs& a_in, int groups, bool tf32, cudaStream_
     }
   }
   const long long mt = (a.M + 127) / 128, nt64 = (a.N + 63) / 64, nt128 = (a.N + 127) / 128;
-  const long long big = (tc ? nt128 : nt64) * mt * groups;
-  if (big >= (tc ? GEM_TF32_BIG_TILE_BLOCKS : GEM_SIMT_BIG_TILE_BLOCKS) * kSmCountHint) {
-    if (tc)
-      launch_mma<128, AK, BK_, EPI>(a, groups, st);
-    else
-      launch_tile<128, AK, BK_, EPI>(a, groups, tf32, st);
+  if (nt128 * mt * groups >= GEM_TF32_BIG_TILE_BLOCKS * kSmCountHint) {
+    launch_mma<128, AK, BK_, EPI>(a, groups, st);
     return cudaGetLastError();
   }
-  const long long small = tc ? nt64 * mt * groups : nt64 * ((a.M + 63) / 64) * groups;
+  const long long small = nt64 * mt * groups;
   int split = 1;
   const long long mn = (long long)a.M * a.N * groups;
-  const int min_chunk = tc ? GEM_TF32_MIN_CHUNK : GEM_SIMT_MIN_CHUNK;   // the tensor cores get through K faster
   if (a.ws && a.M <= 128)
-    while (split < kMaxSplit && small * split < 4 * kSmCountHint && a.K / (2 * split) >= min_chunk &&
+    while (split < kMaxSplit && small * split < 4 * kSmCountHint && a.K / (2 * split) >= GEM_TF32_MIN_CHUNK &&
            mn * 2 * split <= a.ws_floats)
       split *= 2;
   if (split > 1) {
     a.ksplit = split;
     a.kchunk = ((a.K + split - 1) / split + BK - 1) / BK * BK;
   }
-  if (tc)
-    launch_mma<64, AK, BK_, EPI>(a, groups * split, st);
-  else
-    launch_tile<64, AK, BK_, EPI>(a, groups * split, tf32, st);
-  if (split > 1) {
-    // float4 columns when every row of every array starts on a 16-byte boundary
-    auto al = [](const void* ptr, long long stride) {
-      return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0 && stride % 4 == 0;
-    };
-    const bool vec = a.N % 4 == 0 && al(a.C, a.c_group_stride) && a.ldc % 4 == 0 &&
-                     (!(EPI == kBias || EPI == kBiasRelu) || al(a.bias, a.bias_group_stride)) &&
-                     (EPI != kMask || (al(a.mask, a.mask_group_stride) && a.ldmask % 4 == 0));
-    const int V = vec ? 4 : 1;
-    dim3 grid(unsigned((a.N + 256 * V - 1) / (256 * V)), unsigned(a.M * groups));
-    if (vec)
-      gem::launch_pdl(splitk_reduce_kernel<EPI, 4>, grid, 256, 0, st, a);
-    else
-      gem::launch_pdl(splitk_reduce_kernel<EPI, 1>, grid, 256, 0, st, a);
-  }
+  launch_mma<64, AK, BK_, EPI>(a, groups * split, st);
+  if (split > 1) launch_reduce<EPI>(a, groups, st);
   return cudaGetLastError();
 }
 
@@ -1162,7 +1462,11 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   auto act = [&](int l) -> float* { return l == 0 ? scr + M->off_x : scr + M->off_act[l]; };
 
   int rc = GEM_OK;
-  if (!M->external_input) {
+  // the minibatch rows: read in place by the small products of the first layer (its forward
+  // product and its weight gradient have the same size), gathered for the others (rounded for
+  // the tensor cores)
+  const bool in_place = !M->external_input && !tf32 && small_product(b, M->dims[1], M->dims[0], G) ;
+  if (!M->external_input && !in_place) {
     gem::launch_pdl(gather_rows_kernel, dim3(b, G), 256, 0, st, M->X, M->dims[0], batch_rows, b,
                                                    scr + M->off_x, S, tf32 ? 1 : 0);
     if ((rc = cuda_rc(cudaGetLastError()))) return rc;
@@ -1174,6 +1478,7 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   for (int g = 0; g < G; ++g) a.workers[g] = workers[g];
   a.ws = M->ws;
   a.ws_floats = M->ws_floats;
+  a.can_split = b <= 128 && M->scratch_end != nullptr;
   a.status = M->tc_status;
   const long long wstride = (long long)h->stride;
   // floats addressable from p when it lies in the scratch or in the snapshots (0 otherwise)
@@ -1240,8 +1545,8 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   for (int l = 0; l < L; ++l) {
     const int din = M->dims[l], dout = M->dims[l + 1];
     a.M = b; a.N = dout; a.K = din;
-    a.A = Operand{act(l), S, din, 0};
-    a.B = Operand{h->s + M->w_off[l], wstride, din, 1};
+    a.A = l == 0 && in_place ? Operand{M->X, 0, din, 0, batch_rows, b} : Operand{act(l), S, din, 0, nullptr, 0};
+    a.B = Operand{h->s + M->w_off[l], wstride, din, 1, nullptr, 0};
     a.bias = h->s + M->b_off[l];
     a.bias_group_stride = wstride;
     const bool last = l == L - 1;
@@ -1313,7 +1618,10 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
     w.C = grads + M->w_off[l];
     w.c_group_stride = grad_stride;
     w.ldc = din;
-    if (two_streams) w.ws = nullptr;
+    if (two_streams) {
+      w.ws = nullptr;
+      w.can_split = 0;
+    }
     w.bias = nullptr;
     w.mask = nullptr;
     cudaError_t ew;
@@ -1321,15 +1629,15 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
       // D_{l+1}^T, on the weight-gradient stream (the input-gradient chain goes on)
       if ((rc = transpose(wst, scr + M->off_delta[l + 1], S, false, scr + M->off_deltaT[l + 1], b, dout)))
         return rc;
-      w.A = Operand{scr + M->off_deltaT[l + 1], S, b, 0};
-      w.B = Operand{scr + M->off_actT[l], S, b, 0};
+      w.A = Operand{scr + M->off_deltaT[l + 1], S, b, 0, nullptr, 0};
+      w.B = Operand{scr + M->off_actT[l], S, b, 0, nullptr, 0};
       w.a_rounded = 1;
       w.b_rounded = 1;
       set_extents(w, G);
       ew = launch_gemm<true, true, kStore>(w, G, tf32, wst);
     } else {
-      w.A = Operand{scr + M->off_delta[l + 1], S, dout, 0};
-      w.B = Operand{act(l), S, din, 0};
+      w.A = Operand{scr + M->off_delta[l + 1], S, dout, 0, nullptr, 0};
+      w.B = l == 0 && in_place ? Operand{M->X, 0, din, 0, batch_rows, b} : Operand{act(l), S, din, 0, nullptr, 0};
       w.a_rounded = 0;
       w.b_rounded = 0;
       set_extents(w, G);
@@ -1341,8 +1649,8 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
       if (!M->input_grad) break;
       // D_0 = D_1 W_0, the gradient with respect to the input rows (no activation here)
       a.M = b; a.N = din; a.K = dout;
-      a.A = Operand{scr + M->off_delta[1], S, dout, 0};
-      a.B = Operand{h->s + M->w_off[0], wstride, din, 1};
+      a.A = Operand{scr + M->off_delta[1], S, dout, 0, nullptr, 0};
+      a.B = Operand{h->s + M->w_off[0], wstride, din, 1, nullptr, 0};
       a.C = scr + M->off_delta[0];
       a.c_group_stride = S;
       a.ldc = din;
@@ -1355,14 +1663,14 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
     }
     // D_l = (D_{l+1} W_l) * [A_l > 0]: (m = r, k = o) from D, (k = o, n = j) from W_l [dout x din]
     a.M = b; a.N = din; a.K = dout;
-    a.A = Operand{scr + M->off_delta[l + 1], S, dout, 0};
+    a.A = Operand{scr + M->off_delta[l + 1], S, dout, 0, nullptr, 0};
     a.C = scr + M->off_delta[l];
     a.c_group_stride = S;
     a.ldc = din;
     a.mask = act(l);
     a.mask_group_stride = S;
     a.ldmask = din;
-    a.B = Operand{h->s + M->w_off[l], wstride, din, 1};
+    a.B = Operand{h->s + M->w_off[l], wstride, din, 1, nullptr, 0};
     a.bias = nullptr;
     a.a_rounded = 0;
     a.b_rounded = 0;
