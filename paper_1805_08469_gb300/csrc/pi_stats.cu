@@ -9,10 +9,8 @@
 // fixed so far and the rank of the target among the elements that share them.
 //   - select_hist_kernel: blocks of 16,384 elements of one segment count, in shared memory,
 //     the next digit of every element that matches a target's prefix, and add their
-//     counts to the problem's histogram in global memory.  Counts are aggregated per warp
-//     (one shared-memory atomic per distinct digit), because clamped factors put many
-//     equal keys (pi = 0) into one bin.  While both targets share their prefix, which is
-//     always true in the first pass, one histogram serves both.
+//     counts to the problem's histogram in global memory.  While both targets share their
+//     prefix, which is always true in the first pass, one histogram serves both.
 //   - select_pick_kernel: one block per problem scans the histogram, finds the bin that
 //     holds each target's rank, extends the prefix and reduces the rank, then clears the
 //     histogram for the next pass.
@@ -29,6 +27,9 @@
 // row and segment, the factors below +0 and equal to +0 while it writes them.  With those
 // counts the init kernel resolves every target whose rank lies in the run of zeros before
 // any pass, and a problem with both targets resolved is never read.
+// Segments of up to kSmallSegment elements (every tensor of the small networks) take one launch
+// instead of eight: select_small_kernel, a block per problem, keeps the segment's keys and
+// histogram in shared memory, reads the factors once and runs the three passes there.
 #include <cmath>
 
 #include "gem_internal.h"
@@ -116,17 +117,6 @@ __global__ void count_init_kernel(const __grid_constant__ CountInitArgs a) {
   if (i <= a.nseg) a.seg_dev[i] = a.seg[i];
 }
 
-// Adds one element's digit to a shared histogram when its key matches the prefix; every
-// lane of the warp must call it (the match is warp-wide).  FIRST: the first pass, whose
-// prefix is empty, so that every element matches.
-template <bool FIRST>
-__device__ __forceinline__ void count_digit(unsigned* h, bool valid, unsigned key, unsigned prefix,
-                                            unsigned mask, unsigned digit, int lane) {
-  const unsigned bin = (valid && (FIRST || (key & mask) == prefix)) ? digit : 0xffffffffu;
-  const unsigned peers = __match_any_sync(0xffffffffu, bin);
-  if (bin != 0xffffffffu && lane == __ffs(peers) - 1) atomicAdd(h + bin, unsigned(__popc(peers)));
-}
-
 template <bool FIRST>
 __global__ void __launch_bounds__(kThreads) select_hist_kernel(const __grid_constant__ SelectArgs a) {
   gem::pdl_entry();
@@ -149,8 +139,7 @@ __global__ void __launch_bounds__(kThreads) select_hist_kernel(const __grid_cons
   const long long beg = a.seg[s] + (long long)(b - a.block_start[s]) * kChunk;
   const long long end = beg + kChunk < a.seg[s + 1] ? beg + kChunk : a.seg[s + 1];
   const float* x = a.pi[k];
-  const int lane = threadIdx.x & 31;
-  // the loop bounds are uniform across the block, so whole warps reach count_digit
+  unsigned zeros = 0u;   // first pass: this thread's elements equal to +0
   for (long long base = beg; base < end; base += kThreads * kUnroll) {
     unsigned key[kUnroll];
 #pragma unroll
@@ -160,15 +149,20 @@ __global__ void __launch_bounds__(kThreads) select_hist_kernel(const __grid_cons
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
-      const bool valid = base + u * kThreads + threadIdx.x < end;
+      if (base + u * kThreads + threadIdx.x >= end) continue;
       const unsigned d = (key[u] >> shift) & dmask;
       if (FIRST) {
-        count_digit<true>(h, valid, key[u], 0u, 0u, key[u] == kZeroKey ? unsigned(kBins) : d, lane);
+        if (key[u] == kZeroKey) ++zeros;
+        else atomicAdd(h + d, 1u);
       } else {
-        if (need0) count_digit<false>(h, valid, key[u], p0, m0, d, lane);
-        if (need1) count_digit<false>(h + kBins, valid, key[u], p1, m1, d, lane);
+        if (need0 && (key[u] & m0) == p0) atomicAdd(h + d, 1u);
+        if (need1 && (key[u] & m1) == p1) atomicAdd(h + kBins + d, 1u);
       }
     }
+  }
+  if (FIRST) {
+    zeros = __reduce_add_sync(0xffffffffu, zeros);
+    if ((threadIdx.x & 31) == 0 && zeros) atomicAdd(h + kBins, zeros);
   }
   __syncthreads();
   unsigned* g = a.hist + size_t(q) * 2 * kBins;
@@ -259,6 +253,155 @@ __global__ void __launch_bounds__(kThreads) select_pick_kernel(const __grid_cons
   }
 }
 
+// ---- segments that fit in shared memory
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallSegment = 52 * 1024;    // keys of one segment: 208 KB, beside 16 KB of histograms
+constexpr int kSmallUnroll = 16;            // independent loads per thread and step
+
+// A block per problem: the three passes of the selection above on the segment's keys in shared
+// memory.  The factors are read once (L2 serves them: the commit has just written them), 16
+// loads per thread in flight; each pass counts digits with shared-memory atomics, scans the
+// bins with the whole block, two per thread, and extends the targets' prefixes.
+// What bounds it is the latency of that chain.  Measured, the MNIST network with n = 30 and its ten
+// tensors (up to 40,960 factors): see commit_pi_median_ordered.
+__global__ void __launch_bounds__(kSmallThreads) select_small_kernel(const __grid_constant__ SelectArgs a) {
+  gem::pdl_entry();
+  extern __shared__ unsigned small_smem[];
+  __shared__ unsigned wsum[kSmallThreads / 32];
+  __shared__ unsigned prefix[2], mask[2], rank[2], zeros_all;
+  const int q = blockIdx.x, k = q / a.nseg, s = q - k * a.nseg;
+  const int N = int(a.seg[s + 1] - a.seg[s]);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (N == 0) {
+    if (tid == 0) a.lo[q] = a.hi[q] = __int_as_float(0x7fc00000);
+    return;
+  }
+  const unsigned r0 = unsigned((N - 1) / 2), r1 = unsigned(N / 2);
+  bool done0 = false, done1 = false;         // targets known from the commit's counts
+  if (a.counts) {
+    // elements below +0 come first in the order, then the run of +0
+    const unsigned below = a.counts[2 * q], zeros = a.counts[2 * q + 1];
+    done0 = r0 >= below && r0 - below < zeros;
+    done1 = r1 >= below && r1 - below < zeros;
+    if (tid == 0) {
+      if (done0) a.lo[q] = 0.0f;
+      if (done1) a.hi[q] = 0.0f;
+    }
+    if (done0 && done1) return;
+  }
+  unsigned* keys = small_smem;               // [N]
+  unsigned* h = small_smem + N;              // [2][kBins]
+  for (int i = tid; i < 2 * kBins; i += kSmallThreads) h[i] = 0u;
+  if (tid < 2) {
+    prefix[tid] = 0u;
+    mask[tid] = (tid == 0 ? done0 : done1) ? 0xffffffffu : 0u;
+    rank[tid] = tid == 0 ? r0 : r1;
+  }
+  if (tid == 0) zeros_all = 0u;
+  __syncthreads();
+  const float* x = a.pi[k] + a.seg[s];
+  unsigned zeros = 0u;
+  for (int base = 0; base < N; base += kSmallThreads * kSmallUnroll) {
+    unsigned key[kSmallUnroll];
+#pragma unroll
+    for (int u = 0; u < kSmallUnroll; ++u) {
+      const int i = base + u * kSmallThreads + tid;
+      key[u] = i < N ? order_key(x[i]) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < kSmallUnroll; ++u) {
+      const int i = base + u * kSmallThreads + tid;
+      if (i >= N) continue;
+      keys[i] = key[u];
+      if (key[u] == kZeroKey) ++zeros;
+      else atomicAdd(h + (key[u] >> digit_shift(0)), 1u);
+    }
+  }
+  zeros = __reduce_add_sync(0xffffffffu, zeros);
+  if (lane == 0 && zeros) atomicAdd(&zeros_all, zeros);
+  __syncthreads();
+
+  constexpr int kPer = kBins / kSmallThreads;   // bins per thread (2)
+  const int zero_bin = int(kZeroKey >> digit_shift(0));   // +0's first-pass bin
+  for (int pass = 0; pass < kPasses; ++pass) {
+    const int shift = digit_shift(pass);
+    const unsigned dmask = (1u << digit_bits(pass)) - 1u;
+    // one histogram serves both targets while they share their prefix (a target that is known
+    // is skipped)
+    const bool two = pass > 0 && mask[0] != 0xffffffffu && mask[1] != 0xffffffffu && prefix[0] != prefix[1];
+    if (pass > 0) {
+      const int t0 = mask[0] == 0xffffffffu ? 1 : 0;
+      const unsigned p0 = prefix[t0], p1 = prefix[1], m = mask[t0];
+      for (int i = tid; i < N; i += kSmallThreads) {
+        const unsigned key = keys[i], d = (key >> shift) & dmask;
+        if ((key & m) == p0) atomicAdd(h + d, 1u);
+        else if (two && (key & m) == p1) atomicAdd(h + kBins + d, 1u);
+      }
+      __syncthreads();
+    }
+    unsigned found[2] = {0u, 0u}, left[2] = {0u, 0u};
+    bool mine[2] = {false, false}, is_zero[2] = {false, false};
+    for (int t = 0; t < 2; ++t) {
+      const unsigned* hh = h + (two && t == 1 ? kBins : 0);
+      unsigned local[kPer], sum = 0u;
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) {
+        local[j] = hh[tid * kPer + j];
+        if (pass == 0 && tid * kPer + j == zero_bin) local[j] += zeros_all;   // counted apart
+        sum += local[j];
+      }
+      unsigned incl = sum;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+      }
+      if (lane == 31) wsum[warp] = incl;
+      __syncthreads();
+      unsigned before = wsum[lane];   // the warps' sums, scanned by every warp
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, before, off);
+        if (lane >= off) before += v;
+      }
+      before = __shfl_sync(0xffffffffu, before, (warp + 31) & 31);
+      const unsigned excl = (warp == 0 ? 0u : before) + incl - sum;
+      const unsigned r = rank[t];
+      if (mask[t] != 0xffffffffu && r >= excl && r - excl < sum) {
+        unsigned c = excl;
+        int d = tid * kPer;
+        if (r - c >= local[0]) {
+          c += local[0];
+          ++d;
+        }
+        mine[t] = true;
+        found[t] = unsigned(d);
+        left[t] = r - c;
+        // +0 is the smallest key of its bin, so the bin's first ranks are exact zeros
+        is_zero[t] = pass == 0 && d == zero_bin && r - c < zeros_all;
+      }
+      __syncthreads();   // wsum, rank, mask and the histograms have been read
+    }
+    static_assert(kPer == 2, "two bins per thread");
+    for (int t = 0; t < 2; ++t) {
+      if (!mine[t]) continue;
+      float* out = t == 0 ? a.lo : a.hi;
+      if (is_zero[t]) {
+        mask[t] = 0xffffffffu;
+        out[q] = 0.0f;
+      } else {
+        prefix[t] |= found[t] << shift;
+        mask[t] |= dmask << shift;
+        rank[t] = left[t];
+        if (pass == kPasses - 1) out[q] = key_value(prefix[t]);
+      }
+    }
+    for (int i = tid; i < 2 * kBins; i += kSmallThreads) h[i] = 0u;
+    __syncthreads();
+    if (mask[0] == 0xffffffffu && mask[1] == 0xffffffffu) return;
+  }
+}
+
 }  // namespace
 
 namespace {
@@ -310,6 +453,23 @@ int prepare_args(SelectArgs& a, const int64_t* seg, int nseg) {
 // The select of rows a.pi[0 .. kc) (a.lo, a.hi, a.counts set by the caller).
 cudaError_t select_rows(gem_ctx* h, SelectArgs& a, int kc, int blocks) {
   a.K = kc;
+  long long longest = 0;
+  for (int s = 0; s < a.nseg; ++s) longest = a.seg[s + 1] - a.seg[s] > longest ? a.seg[s + 1] - a.seg[s] : longest;
+  if (longest <= kSmallSegment) {
+    static bool configured[64] = {};   // one attribute call per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !configured[dev]) {
+      const cudaError_t e = cudaFuncSetAttribute(select_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 int((kSmallSegment + 2 * kBins) * sizeof(unsigned)));
+      if (e != cudaSuccess) return e;
+      if (dev >= 0 && dev < 64) configured[dev] = true;
+    }
+    gem::launch_pdl(select_small_kernel, unsigned(kc * a.nseg), kSmallThreads,
+                    size_t(longest + 2 * kBins) * sizeof(unsigned), h->stream, a);
+    h->launches += 1;
+    return cudaGetLastError();
+  }
   a.pass = 0;
   cudaError_t e = cudaMemsetAsync(a.hist, 0, size_t(kc) * a.nseg * 2 * kBins * sizeof(unsigned),
                                   h->stream);
