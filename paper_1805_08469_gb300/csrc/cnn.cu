@@ -469,16 +469,27 @@ __global__ void __launch_bounds__(kThreads) conv_finish_kernel(const __grid_cons
   const long long e = q % (n1 + n2);
   float* grad = a.grads + g * a.grad_stride;
   const float* slot = a.scr + g * a.S;
-  float acc = 0.f;
+  // kAhead samples' partials in flight, added in sample order
+  constexpr int kAhead = 16;
+  auto sum = [&](const float* part, long long ld) {
+    float acc = 0.f;
+    for (int i0 = 0; i0 < a.b; i0 += kAhead) {
+      float v[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) v[u] = i0 + u < a.b ? part[(i0 + u) * ld] : 0.f;
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if (i0 + u < a.b) acc += v[u];
+    }
+    return acc;
+  };
   if (e < n1) {
     const int co = int(e / per1), k = int(e % per1);
-    for (int i = 0; i < a.b; ++i) acc += slot[a.o_p1 + ((long long)i * a.c1 + co) * per1 + k];
-    grad[k < per1 - 1 ? a.w1 + co * (per1 - 1) + k : a.b1 + co] = acc;
+    grad[k < per1 - 1 ? a.w1 + co * (per1 - 1) + k : a.b1 + co] = sum(slot + a.o_p1 + co * per1 + k, n1);
   } else {
     const long long e2 = e - n1;
     const int co = int(e2 / per2), k = int(e2 % per2);
-    for (int i = 0; i < a.b; ++i) acc += slot[a.o_p2 + ((long long)i * a.c2 + co) * per2 + k];
-    grad[k < per2 - 1 ? a.w2 + (long long)co * (per2 - 1) + k : a.b2 + co] = acc;
+    grad[k < per2 - 1 ? a.w2 + (long long)co * (per2 - 1) + k : a.b2 + co] = sum(slot + a.o_p2 + co * per2 + k, n2);
   }
 }
 

@@ -941,14 +941,15 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constan
 // Products with few outputs per row (N <= kMaxClasses), used for the logits:
 // C[g][m][n] = sum_k A[g][m][k] B[g][n][k] + bias[n], A and B K-major.  The block first
 // copies the worker's B (N x K, TF32-rounded when asked) into shared memory; then each warp
-// takes whole rows m: lane l accumulates k = l, l + 32, ... (coalesced A reads, conflict-free
-// shared reads), a fixed butterfly adds the 32 lane sums, and lane 0 writes the N outputs
-// of the row.  Deterministic.  rows_per_block rows per block; NC >= N classes compiled in
+// takes whole rows m: lane l accumulates k = l, l + 32, ... (coalesced A reads, 16 in flight;
+// conflict-free shared reads), a fixed butterfly adds the 32 lane sums, and lane n takes output
+// n of the row.  Deterministic.  rows_per_block rows per block; NC >= N classes compiled in
 // (16 or 32), so that a network with few classes carries no idle class slots.
-// The last layer's softmax cross-entropy, fused into the logits kernel (XENT): the lane
-// that finishes a row's logits z goes on, with the operations and order of
-// softmax_xent_kernel, to the row's loss gradient (softmax(z) - onehot(y)) / b and its
-// loss; the row losses are summed in row order by bias_grad_kernel.
+// Latency bounds it (a warp has one row or a few).
+// The last layer's softmax cross-entropy, fused into the logits kernel (XENT): lane n goes on
+// from the logit z_n, with the operations and order of softmax_xent_kernel, to its element of
+// the row's loss gradient (softmax(z) - onehot(y)) / b, and lane 0 to the row's loss; the row
+// losses are summed in row order by bias_grad_kernel.
 struct XentArgs {
   const int32_t* labels;        // [rows of the data set]
   const int32_t* batch_rows;    // [groups][b]
@@ -959,7 +960,7 @@ struct XentArgs {
 };
 
 template <bool TF32, bool XENT, int NC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 gemm_small_n_kernel(const __grid_constant__ GemmArgs p, int rows_per_block,
                     const __grid_constant__ XentArgs x) {
   gem::pdl_entry();
@@ -970,6 +971,21 @@ gemm_small_n_kernel(const __grid_constant__ GemmArgs p, int rows_per_block,
   const float* B = p.B.base + (p.B.by_worker ? (long long)p.workers[g] : (long long)g) * p.B.group_stride;
   const int N = p.N, K = p.K;
   const bool vec = K % 4 == 0 && p.B.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15u) == 0;
+  const int r0 = blockIdx.x * rows_per_block;
+  const int r1 = min(p.M, r0 + rows_per_block);
+  // elements lane, lane + 32, ... of a row of A from k0 on, kAhead in flight; the warp's first row
+  // is on its way while the weights are
+  constexpr int kAhead = 16;
+  float av[kAhead];
+  auto load_row = [&](int m, int k0) {
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int k = k0 + 32 * u + lane;
+      av[u] = k < K ? A[(long long)m * p.A.ld + k] : 0.f;
+    }
+  };
+  const float bias_n = lane < N ? p.bias[(long long)p.workers[g] * p.bias_group_stride + lane] : 0.f;
+  if (r0 + warp < r1) load_row(r0 + warp, 0);
   if (vec) {   // 16-byte asynchronous copies, all in flight at once, then rounded in place
     const int chunks = N * K / 4;
     for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
@@ -996,22 +1012,25 @@ gemm_small_n_kernel(const __grid_constant__ GemmArgs p, int rows_per_block,
     }
   }
   __syncthreads();
-  const float* bias = p.bias + (long long)p.workers[g] * p.bias_group_stride;
-  const int r0 = blockIdx.x * rows_per_block;
-  const int r1 = min(p.M, r0 + rows_per_block);
   for (int m = r0 + warp; m < r1; m += 8) {
-    const float* a = A + (long long)m * p.A.ld;
+    if (m != r0 + warp) load_row(m, 0);
     float acc[NC];
 #pragma unroll
     for (int n = 0; n < NC; ++n) acc[n] = 0.f;
-    constexpr int kUnroll = NC <= 16 ? 8 : 4;   // A loads in flight within the register budget
-#pragma unroll kUnroll
-    for (int k = lane; k < K; k += 32) {
-      const float av = TF32 ? to_tf32(a[k]) : a[k];
+    for (int k0 = 0; k0 < K; k0 += 32 * kAhead) {
+      if (k0 > 0) load_row(m, k0);
 #pragma unroll
-      for (int n = 0; n < NC; ++n)
-        if (n < N) acc[n] = fmaf(av, Bsm[n * K + k], acc[n]);
+      for (int u = 0; u < kAhead; ++u) {
+        const int k = k0 + 32 * u + lane;
+        if (k < K) {
+          const float v = TF32 ? to_tf32(av[u]) : av[u];
+#pragma unroll
+          for (int n = 0; n < NC; ++n)
+            if (n < N) acc[n] = fmaf(v, Bsm[n * K + k], acc[n]);
+        }
+      }
     }
+    // every lane gets the row's sums (the butterfly adds the same pairs in every lane)
 #pragma unroll
     for (int n = 0; n < NC; ++n) {
       if (n < N) {
@@ -1019,42 +1038,35 @@ gemm_small_n_kernel(const __grid_constant__ GemmArgs p, int rows_per_block,
         for (int off = 16; off > 0; off >>= 1) acc[n] += __shfl_xor_sync(0xffffffffu, acc[n], off);
       }
     }
-    if (lane == 0) {
-      float* c = p.C + (long long)g * p.c_group_stride + (long long)m * p.ldc;
+    // lane n goes on with class n
+    float z = 0.f;
 #pragma unroll
-      for (int n = 0; n < NC; ++n)
-        if (n < N) {
-          acc[n] = acc[n] + bias[n];   // the logit z_n
-          c[n] = acc[n];
-        }
-      if (XENT) {
-        int y = x.labels[x.batch_rows[(long long)g * x.b + m]];
-        const bool bad_label = y < 0 || y >= N;   // reported as a NaN loss and gradient
-        if (bad_label) y = 0;
-        float zmax = acc[0];
+    for (int n = 0; n < NC; ++n)
+      if (n < N && lane == n) z = acc[n];
+    const bool mine = lane < N;
+    z = z + bias_n;   // the logit z_n
+    if (mine) p.C[(long long)g * p.c_group_stride + (long long)m * p.ldc + lane] = z;
+    if (XENT) {
+      int y = x.labels[x.batch_rows[(long long)g * x.b + m]];
+      const bool bad_label = y < 0 || y >= N;   // reported as a NaN loss and gradient
+      if (bad_label) y = 0;
+      float zmax = mine ? z : -INFINITY;
 #pragma unroll
-        for (int n = 1; n < NC; ++n)
-          if (n < N) zmax = fmaxf(zmax, acc[n]);
-        float e[NC];
-        float sum = 0.f;
+      for (int off = 16; off > 0; off >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, off));
+      const float e = expf(z - zmax);
+      float sum = 0.f;   // over the classes in order
 #pragma unroll
-        for (int n = 0; n < NC; ++n)
-          if (n < N) {
-            e[n] = expf(acc[n] - zmax);
-            sum += e[n];
-          }
-        const float inv_b = 1.0f / float(x.b);
-        const float poison = bad_label ? __int_as_float(0x7fc00000) : 0.f;
-        float* d = x.delta + (long long)g * x.group_stride + (long long)m * N;
-        float zy = acc[0];
-#pragma unroll
-        for (int n = 0; n < NC; ++n)
-          if (n < N) {
-            d[n] = (e[n] / sum - (n == y ? 1.f : 0.f)) * inv_b + poison;
-            if (n == y) zy = acc[n];
-          }
-        x.row_loss[(long long)g * x.group_stride + m] = (logf(sum) + zmax) - zy + poison;
+      for (int n = 0; n < NC; ++n) {
+        const float en = __shfl_sync(0xffffffffu, e, n);
+        if (n < N) sum += en;
       }
+      const float inv_b = 1.0f / float(x.b);
+      const float poison = bad_label ? __int_as_float(0x7fc00000) : 0.f;
+      if (mine)
+        x.delta[(long long)g * x.group_stride + (long long)m * N + lane] =
+            (e / sum - (lane == y ? 1.f : 0.f)) * inv_b + poison;
+      const float zy = __shfl_sync(0xffffffffu, z, y);
+      if (lane == 0) x.row_loss[(long long)g * x.group_stride + m] = (logf(sum) + zmax) - zy + poison;
     }
   }
 }
@@ -1204,17 +1216,30 @@ __global__ void __launch_bounds__(256)
 bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
                  long long slot_stride, float* grad, long long grad_stride) {
   gem::pdl_entry();
+  constexpr int kAhead = 16;
   __shared__ float part[8][33];
+  __shared__ float row_loss[kMaxBatch];
   const int g = blockIdx.y;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   const int q = blockIdx.x * 32 + x;
+  const bool sums_loss = a.losses && blockIdx.x == 0;
+  if (sums_loss)
+    for (int r = threadIdx.x; r < a.b; r += 256) row_loss[r] = delta[g * slot_stride + a.row_loss_off + r];
   float s = 0.f;
   int l = 0, o = 0;
   if (q < a.first[a.n_layers]) {
     while (q >= a.first[l + 1]) ++l;
     o = q - a.first[l];
-    const float* D = delta + g * slot_stride + a.delta_off[l];
-    for (int r = y; r < a.b; r += 8) s += D[(long long)r * a.width[l] + o];
+    const float* D = delta + g * slot_stride + a.delta_off[l] + o;
+    const long long ld = a.width[l];
+    for (int r0 = y; r0 < a.b; r0 += 8 * kAhead) {   // kAhead rows in flight, added in order
+      float v[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) v[u] = r0 + 8 * u < a.b ? D[(r0 + 8 * u) * ld] : 0.f;
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if (r0 + 8 * u < a.b) s += v[u];
+    }
   }
   part[y][x] = s;
   __syncthreads();
@@ -1224,10 +1249,9 @@ bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
     for (int w = 0; w < 8; ++w) t += part[w][x];
     grad[g * grad_stride + a.grad_off[l] + o] = t;
   }
-  if (a.losses && blockIdx.x == 0 && threadIdx.x == 0) {   // the minibatch loss, rows in order
-    const float* rl = delta + g * slot_stride + a.row_loss_off;
+  if (sums_loss && threadIdx.x == 0) {   // the minibatch loss, rows in order
     float t = 0.f;
-    for (int r = 0; r < a.b; ++r) t += rl[r];
+    for (int r = 0; r < a.b; ++r) t += row_loss[r];
     a.losses[g] = t / float(a.b);
   }
 }
