@@ -1,6 +1,6 @@
 // Grouped TF32 products on the tcgen05 tensor cores, the accumulator in tensor memory.
 //
-// A persistent kernel: one CTA per SM walks the 128 x BN output tiles t = blockIdx.x,
+// A persistent kernel: one CTA per SM walks the 128 x BN (BN = 64, 96 or 128) output tiles t = blockIdx.x,
 // blockIdx.x + gridDim.x, ... of all groups (the workers of a segment), in k-blocks of 32
 // fp32 values (128 bytes per operand row).  Its warps have four roles that meet only at
 // shared-memory barriers, so that the copies, the MMAs and the epilogue of consecutive
@@ -72,7 +72,7 @@ struct Cfg {
   static constexpr int kEpiAt = kStages * kStage;      // 8 warps x 32 x 33 floats
   static constexpr int kBarrierAt = kEpiAt + 8 * 32 * 33 * 4;
   static constexpr int kSmem = kBarrierAt + 512 + 1024;   // barriers, slots; alignment slack
-  static constexpr int kTmemCols = 2 * BN;             // two accumulators
+  static constexpr int kTmemCols = BN == 64 ? 128 : 256;   // two accumulators, allocated as a power of 2
 };
 
 // Kernel parameters: the product and the tensor maps of its operands (64-byte aligned, in
@@ -708,9 +708,15 @@ cudaError_t launch(const Args& a, int groups, bool a_kmajor, bool b_kmajor, int 
   // work for 4/3 of the bytes); otherwise 64-wide, which spreads a product with few tiles
   // (a 128-row minibatch panel per worker) over more SMs: its weights come from DRAM, and
   // more SMs pulling them finish sooner than fewer copying fewer bytes each (measured: the
-  // forward products of a 13-worker segment 29.7 us 64-wide, 36 us 128-wide)
-  const long long tiles128 = (long long)((a.N + 127) / 128) * ((a.M + kBM - 1) / kBM) * groups;
-  if (tiles128 >= 152) return launch_cfg<128>(a, groups, epi, stream);
+  // forward products of a 13-worker segment 29.7 us 64-wide, 36 us 128-wide); or 96-wide where
+  // the busiest SM then copies fewer bytes: 1,000 columns of 13 workers are 208 tiles 64-wide,
+  // two on most of 152 SMs and one on the others, and 143 tiles 96-wide, one each (forward
+  // 34.8 -> 30.9 us, a segment's gradients 351 -> 338 us, the whole run 2,265 -> 2,217 us)
+  const long long panels = (long long)((a.M + kBM - 1) / kBM) * groups;
+  auto tiles = [&](int bn) { return (a.N + bn - 1) / bn * panels; };
+  if (tiles(128) >= 152) return launch_cfg<128>(a, groups, epi, stream);
+  auto bytes = [&](int bn) { return (tiles(bn) + 151) / 152 * (kBM + bn); };   // of the busiest SM's copies
+  if (bytes(96) < bytes(64)) return launch_cfg<96>(a, groups, epi, stream);
   return launch_cfg<64>(a, groups, epi, stream);
 }
 
