@@ -38,6 +38,7 @@ using gem::mlp::kMaxGroups;
 constexpr int kK = 5;  // kernel side
 constexpr int kThreads = 256;
 constexpr long long kMaxSampleSmem = 160 * 1024;   // per-sample staging, bytes
+constexpr long long kMaxSmem28 = 200 * 1024;       // the same of the kernels for the paper's map sizes
 
 struct Shape {
   int H, c1, c2, f1, f2, C;
@@ -143,15 +144,13 @@ __device__ __forceinline__ void stage_wait() {
 }
 
 // conv1 + bias, 2 x 2 max-pool, ReLU: thread per pooled output (co, py, px), the 6 x 6
-// input patch of its window and the channel's 25 weights in registers.  HC: the input side
-// when known at compile time (the paper's network: 28), 0 reads it from the arguments.
-template <int HC>
+// input patch of its window and the channel's 25 weights in registers.
 __global__ void __launch_bounds__(kThreads) conv1_pool_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ float sm[];
   const long long gi = blockIdx.x;
   const int g = int(gi / a.b), i = int(gi % a.b);
-  const int H = HC ? HC : a.H, H1 = H - (kK - 1), P1 = H1 / 2;
+  const int H = a.H, H1 = H - (kK - 1), P1 = H1 / 2;
   const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
   float* xs = sm;                                   // [H * H]
   float* ws = xs + H * H;                           // [c1][25]
@@ -189,16 +188,14 @@ __global__ void __launch_bounds__(kThreads) conv1_pool_kernel(const __grid_const
 
 // conv2 + bias, dropout scale, 2 x 2 max-pool, ReLU -> the head's features: thread per
 // pooled output (co, py, px), per input channel the 6 x 6 patch of its window and the 25
-// weights in registers.  P1C: conv1's pooled side when known at compile time (12), 0 reads
-// it from the arguments.
+// weights in registers.
 constexpr int kPool2Threads = 320;
-template <int P1C>
 __global__ void __launch_bounds__(kPool2Threads) conv2_pool_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ float sm[];
   const long long gi = blockIdx.x;
   const int g = int(gi / a.b), i = int(gi % a.b);
-  const int P1 = P1C ? P1C : a.P1, H2 = P1 - (kK - 1), P2 = H2 / 2;
+  const int P1 = a.P1, H2 = P1 - (kK - 1), P2 = H2 / 2;
   const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
   const int n_a1 = a.c1 * P1 * P1, n_w = a.c2 * a.c1 * kK * kK;
   float* a1s = sm;                                  // [c1][P1][P1]
@@ -272,19 +269,15 @@ __global__ void __launch_bounds__(kThreads) pool2_back_kernel(const __grid_const
 // which spreads the rows that one warp reads over distinct banks.
 constexpr int kBackRow = 12;
 constexpr int kBackThreads = 128;
-// H2C, P1C: conv2's output side and conv1's pooled side when known at compile time (the
-// paper's network: 8 and 12), which folds the column bounds; 0 reads them from the
-// arguments.  Threads take channels fastest, so the lanes of a warp share a few output
-// rows: they read the same dz2 row stretch (a shared-memory broadcast) and skip the same
-// kernel rows.
-template <int H2C, int P1C>
+// Threads take channels fastest, so the lanes of a warp share a few output rows: they read the
+// same dz2 row stretch (a shared-memory broadcast) and skip the same kernel rows.
 __global__ void __launch_bounds__(kBackThreads) conv2_back_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ float sm[];
   const long long gi = blockIdx.x;
   const int g = int(gi / a.b), i = int(gi % a.b);
   const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
-  const int H2 = H2C ? H2C : a.H2, P1 = P1C ? P1C : a.P1, pitch = H2 + 1;
+  const int H2 = a.H2, P1 = a.P1, pitch = H2 + 1;
   const int n_dz2 = a.c2 * H2 * H2, n_w = a.c2 * a.c1 * kK * kK, n_a1 = a.c1 * P1 * P1;
   float* dzs = sm;                                  // [c2][H2][pitch]
   float* ws = dzs + a.c2 * H2 * pitch;              // [c2][c1][25]
@@ -347,14 +340,12 @@ __global__ void __launch_bounds__(kBackThreads) conv2_back_kernel(const __grid_c
 // then columns.  A thread takes the kK weights (co, ci, ky, 0..kK-1) of one kernel row and
 // slides a window of kK input values along each input row (one new load per column); the
 // last c2 work items are the biases.
-// H2C, P1C as in conv2_back_kernel.
-template <int H2C, int P1C>
 __global__ void __launch_bounds__(kThreads) conv2_wpart_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ float sm[];
   const long long gi = blockIdx.x;
   const int g = int(gi / a.b), i = int(gi % a.b);
-  const int H2 = H2C ? H2C : a.H2, P1 = P1C ? P1C : a.P1;
+  const int H2 = a.H2, P1 = a.P1;
   const int n_dz2 = a.c2 * H2 * H2, n_a1 = a.c1 * P1 * P1;
   float* dzs = sm;                                  // [c2][H2][H2]
   float* a1s = dzs + n_dz2;                         // [c1][P1][P1]
@@ -403,16 +394,13 @@ __global__ void __launch_bounds__(kThreads) conv2_wpart_kernel(const __grid_cons
 // Per-sample partial sums of conv1's weight and bias gradients, over the output rows then
 // columns: a thread per kernel row (co, ky) with a sliding window as in conv2_wpart_kernel,
 // then the c1 biases.
-// H1C, HC: conv1's output side and the input side when known at compile time (the
-// paper's network: 24 and 28); 0 reads them from the arguments.
 constexpr int kW1Threads = 64;
-template <int H1C, int HC>
 __global__ void __launch_bounds__(kW1Threads) conv1_wpart_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ float sm[];
   const long long gi = blockIdx.x;
   const int g = int(gi / a.b), i = int(gi % a.b);
-  const int H1 = H1C ? H1C : a.H1, H = HC ? HC : a.H;
+  const int H1 = a.H1, H = a.H;
   const int n_dz1 = a.c1 * H1 * H1;
   float* dzs = sm;                                  // [c1][H1][H1]
   float* xs = dzs + n_dz1;                          // [H][H]
@@ -457,38 +445,413 @@ __global__ void __launch_bounds__(kW1Threads) conv1_wpart_kernel(const __grid_co
   }
 }
 
+// ---- the paper's map sizes (28 -> 24 -> 12 -> 8 -> 4), any channel counts
+//
+// The kernels above read shared memory a word at a time (13 to 61 words per 40 to 100 FMAs), and
+// that bounds them.  With the sizes fixed every row starts on a 16-byte boundary, so rows come
+// as two or three 16-byte reads (or 8-byte ones at even offsets), and a thread keeps what it
+// read for several outputs: all channels of an input patch, two output channels, two rows, four
+// output channels.  A kernel's 25 weights lie at a pitch of 28 floats, read as seven 16-byte words.
+// Every sum keeps the order of the kernels above (a term that they add and these leave out, or
+// the other way round, is an exact zero), so the results are the same bits.
+// The gradient into conv2's output (pool2_back_kernel) is rebuilt from the features where it
+// is needed, and the gradient into conv1's output is kept before its routing, a quarter of the
+// values: conv1_wpart28_kernel routes it on chip.
+// Measured, segments of about 12 workers, b = 64 (launch list, us): conv1_pool 11.8 -> 10.2, conv2_pool
+// 21.5 -> 16.8, pool2_back 5.2 and conv2_back 38.4 -> 26.4, conv2_wpart 24.0 -> 18.8, conv1_wpart 21.7 ->
+// 16.3; the run of n = 100 1,081 -> 847 us.
+constexpr int kH = 28, kH1 = 24, kP1 = 12, kH2 = 8, kP2 = 4;   // map sides
+constexpr int kWPitch = 28;                                    // floats per kernel of 25 weights
+constexpr int kPer28 = 2;                                      // samples per block of conv2_pool28_kernel
+constexpr int kBackPer28 = 3;                                  // the same of conv2_back28_kernel
+// floats between the channels of a map in shared memory where the lanes of a quarter-warp read
+// 16 bytes each of different channels: 576 + 4, and 144 + 12, for which (channel, row) in turn
+// step by 12 floats mod 32; the plain strides gave 7- and 2-way bank conflicts
+constexpr int kDz1Pitch = kH1 * kH1 + 4, kA1Pitch = kP1 * kP1 + 12;
+
+// Start copying n kernels of 25 weights to the pitch of 28.
+__device__ __forceinline__ void stage_kernels(float* dst, const float* src, int n) {
+  for (int q = threadIdx.x; q < n * kK * kK; q += blockDim.x) cp_async4(dst + q / 25 * kWPitch + q % 25, src + q);
+}
+
+__device__ __forceinline__ void load_kernel(float (&w)[kWPitch], const float* src) {
+#pragma unroll
+  for (int v = 0; v < kWPitch / 4; ++v) {
+    const float4 f = reinterpret_cast<const float4*>(src)[v];
+    w[4 * v] = f.x;
+    w[4 * v + 1] = f.y;
+    w[4 * v + 2] = f.z;
+    w[4 * v + 3] = f.w;
+  }
+}
+
+template <int N>
+__device__ __forceinline__ void load_floats(float (&x)[N], const float* src) {
+  static_assert(N % 4 == 0, "16-byte reads");
+#pragma unroll
+  for (int v = 0; v < N / 4; ++v) {
+    const float4 f = reinterpret_cast<const float4*>(src)[v];
+    x[4 * v] = f.x;
+    x[4 * v + 1] = f.y;
+    x[4 * v + 2] = f.z;
+    x[4 * v + 3] = f.w;
+  }
+}
+
+// The 6 x 6 patch at an even column of rows of `ld` floats (even).
+__device__ __forceinline__ void load_patch(float (&x)[kK + 1][kK + 1], const float* src, int ld) {
+#pragma unroll
+  for (int r = 0; r <= kK; ++r)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2 f = *reinterpret_cast<const float2*>(src + r * ld + 2 * c);
+      x[r][2 * c] = f.x;
+      x[r][2 * c + 1] = f.y;
+    }
+}
+
+// conv1 + bias, pool, ReLU: a block per sample, a thread per window (py, px), which keeps its
+// input patch for every channel.
+constexpr int kPool1Threads28 = 160;   // 144 windows
+__global__ void __launch_bounds__(kPool1Threads28) conv1_pool28_kernel(const __grid_constant__ ConvArgs a) {
+  gem::pdl_entry();
+  extern __shared__ __align__(16) float sm[];
+  const long long gi = blockIdx.x;
+  const int g = int(gi / a.b), i = int(gi % a.b);
+  const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
+  float* xs = sm;                                   // [28][28]
+  float* ws = xs + kH * kH;                         // [c1][28]: 25 weights, the bias
+  stage(xs, a.X + (long long)a.rows[gi] * kH * kH, kH * kH);
+  stage_kernels(ws, th + a.w1, a.c1);
+  for (int q = threadIdx.x; q < a.c1; q += blockDim.x) cp_async4(ws + q * kWPitch + 25, th + a.b1 + q);
+  stage_wait();
+  const int t = threadIdx.x;
+  if (t >= kP1 * kP1) return;
+  uint8_t* k1s = reinterpret_cast<uint8_t*>(a.scr + g * a.S + a.o_k1) + (long long)i * a.c1 * kP1 * kP1;
+  float* a1s = a.scr + g * a.S + a.o_a1 + (long long)i * a.c1 * kP1 * kP1;
+  float x[kK + 1][kK + 1];
+  load_patch(x, xs + 2 * (t / kP1) * kH + 2 * (t % kP1), kH);
+  for (int co = 0; co < a.c1; ++co) {
+    float w[kWPitch];
+    load_kernel(w, ws + co * kWPitch);
+    float v[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) v[d] = w[25];
+#pragma unroll
+    for (int ky = 0; ky < kK; ++ky)
+#pragma unroll
+      for (int kx = 0; kx < kK; ++kx)
+#pragma unroll
+        for (int d = 0; d < 4; ++d) v[d] = fmaf(w[ky * kK + kx], x[(d >> 1) + ky][(d & 1) + kx], v[d]);
+    float m;
+    k1s[co * kP1 * kP1 + t] = uint8_t(first_max4(v, &m));
+    a1s[co * kP1 * kP1 + t] = m > 0.f ? m : 0.f;
+  }
+}
+
+// conv2 + bias, dropout scale, pool, ReLU: a block per kPer28 samples of a worker, 16 threads per
+// pair of output channels and sample, a thread per window, which keeps its patch for both.
+constexpr int kPool2Threads28 = 320;
+__global__ void __launch_bounds__(kPool2Threads28) conv2_pool28_kernel(const __grid_constant__ ConvArgs a) {
+  gem::pdl_entry();
+  extern __shared__ __align__(16) float sm[];
+  const int per_g = (a.b + kPer28 - 1) / kPer28;
+  const int g = blockIdx.x / per_g, i0 = (blockIdx.x - g * per_g) * kPer28;
+  const int ns = min(kPer28, a.b - i0);
+  const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
+  const int n_a1 = a.c1 * kP1 * kP1;
+  float* ws = sm;                                   // [c2][c1][28]
+  float* a1s = ws + a.c2 * a.c1 * kWPitch;          // [kPer28][c1][12][12]
+  stage(a1s, a.scr + g * a.S + a.o_a1 + (long long)i0 * n_a1, ns * n_a1);
+  stage_kernels(ws, th + a.w2, a.c2 * a.c1);
+  stage_wait();
+  const int pairs = (a.c2 + 1) / 2;
+  for (int q = threadIdx.x; q < ns * pairs * kP2 * kP2; q += blockDim.x) {
+    const int px = q % kP2, py = q / kP2 % kP2, cp = q / (kP2 * kP2) % pairs, si = q / (kP2 * kP2 * pairs);
+    const int i = i0 + si, co0 = 2 * cp, co1 = min(co0 + 1, a.c2 - 1);
+    const long long gi = (long long)g * a.b + i;
+    float v[2][4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+      v[0][d] = th[a.b2 + co0];
+      v[1][d] = th[a.b2 + co1];
+    }
+    const float* in = a1s + si * n_a1 + 2 * py * kP1 + 2 * px;
+    const float* w0p = ws + co0 * a.c1 * kWPitch;
+    const float* w1p = ws + co1 * a.c1 * kWPitch;
+    for (int ci = 0; ci < a.c1; ++ci) {
+      float x[kK + 1][kK + 1], w0[kWPitch], w1[kWPitch];
+      load_patch(x, in + ci * kP1 * kP1, kP1);
+      load_kernel(w0, w0p + ci * kWPitch);
+      load_kernel(w1, w1p + ci * kWPitch);
+#pragma unroll
+      for (int ky = 0; ky < kK; ++ky)
+#pragma unroll
+        for (int kx = 0; kx < kK; ++kx)
+#pragma unroll
+          for (int d = 0; d < 4; ++d) {
+            v[0][d] = fmaf(w0[ky * kK + kx], x[(d >> 1) + ky][(d & 1) + kx], v[0][d]);
+            v[1][d] = fmaf(w1[ky * kK + kx], x[(d >> 1) + ky][(d & 1) + kx], v[1][d]);
+          }
+    }
+    uint8_t* k2 = reinterpret_cast<uint8_t*>(a.scr + g * a.S + a.o_k2) + (long long)i * a.c2 * kP2 * kP2;
+    float* feat = a.head + g * a.head_S + a.head_x + (long long)i * a.F;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int co = co0 + e;
+      if (co >= a.c2) break;
+      const float s = a.drop[gi * a.c2 + co];
+#pragma unroll
+      for (int d = 0; d < 4; ++d) v[e][d] = v[e][d] * s;   // dropout: the channel's scale
+      float m;
+      k2[co * kP2 * kP2 + py * kP2 + px] = uint8_t(first_max4(v[e], &m));
+      feat[co * kP2 * kP2 + py * kP2 + px] = m > 0.f ? m : 0.f;
+    }
+  }
+}
+
+// The gradient into conv2's (pre-dropout) output of one sample, as pool2_back_kernel makes it,
+// to dst [c2][8][8] in shared memory.
+__device__ __forceinline__ void rebuild_dz2(float* dst, const ConvArgs& a, int g, int i) {
+  const long long gi = (long long)g * a.b + i;
+  const float* feat = a.head + g * a.head_S + a.head_x + (long long)i * a.F;
+  const float* dfeat = a.head + g * a.head_S + a.head_dx + (long long)i * a.F;
+  const uint8_t* k2 = reinterpret_cast<const uint8_t*>(a.scr + g * a.S + a.o_k2) + (long long)i * a.c2 * kP2 * kP2;
+  for (int q = threadIdx.x; q < a.c2 * kP2 * kP2; q += blockDim.x) {
+    const int px = q % kP2, py = q / kP2 % kP2, co = q / (kP2 * kP2);
+    const float v = feat[q] > 0.f ? dfeat[q] * a.drop[gi * a.c2 + co] : 0.f;
+    const int am = k2[q];
+    float* d = dst + (co * kH2 + 2 * py) * kH2 + 2 * px;
+    *reinterpret_cast<float2*>(d) = make_float2(am == 0 ? v : 0.f, am == 1 ? v : 0.f);
+    *reinterpret_cast<float2*>(d + kH2) = make_float2(am == 2 ? v : 0.f, am == 3 ? v : 0.f);
+  }
+}
+
+// Gradient with respect to conv1's pooled outputs through the ReLU mask, before its routing
+// through pool1: a block per kBackPer28 samples, a thread per sample, input channel and pair of
+// rows (py0, py0 + 1): the kernel's 25 weights and each row of dz2 are read once for both.
+// The rows y of dz2 come from py0 + 1 down, so that each output row adds its kernel rows
+// from 0 up.  The threads of a warp share the pair (samples and channels vary: 30 of 32 lanes
+// for 10 channels), so that a pair near the edge, which meets 2 or 4 rows of dz2 instead of 6,
+// skips the others as a warp.
+constexpr int kBackThreads28 = 192;
+__global__ void __launch_bounds__(kBackThreads28) conv2_back28_kernel(const __grid_constant__ ConvArgs a) {
+  gem::pdl_entry();
+  extern __shared__ __align__(16) float sm[];
+  const int per_g = (a.b + kBackPer28 - 1) / kBackPer28;
+  const int g = blockIdx.x / per_g, i0 = (blockIdx.x - g * per_g) * kBackPer28;
+  const int ns = min(kBackPer28, a.b - i0);
+  const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
+  const int n_dz2 = a.c2 * kH2 * kH2;
+  float* ws = sm;                                   // [c2][c1][28]
+  float* dzs = ws + a.c2 * a.c1 * kWPitch;          // [kBackPer28][c2][8][8]
+  stage_kernels(ws, th + a.w2, a.c2 * a.c1);
+  for (int si = 0; si < ns; ++si) rebuild_dz2(dzs + si * n_dz2, a, g, i0 + si);
+  stage_wait();
+  const int per_pair = (kBackPer28 * a.c1 + 31) / 32 * 32;   // whole warps
+  for (int q = threadIdx.x; q < per_pair * (kP1 / 2); q += blockDim.x) {
+    const int pair = q / per_pair, sc = q - pair * per_pair;
+    const int si = sc / a.c1, ci = sc - si * a.c1, py0 = 2 * pair;
+    if (si >= ns) continue;
+    float acc[2][kP1];
+#pragma unroll
+    for (int j = 0; j < kP1; ++j) acc[0][j] = acc[1][j] = 0.f;
+    for (int co = 0; co < a.c2; ++co) {
+      float w[kWPitch];
+      load_kernel(w, ws + (co * a.c1 + ci) * kWPitch);
+      const float* dz = dzs + si * n_dz2 + co * kH2 * kH2;
+#pragma unroll
+      for (int t = 0; t <= kK; ++t) {   // y = py0 + 1 - t: kernel row t of output row py0 + 1, t - 1 of py0
+        const int y = py0 + 1 - t;
+        if (y < 0 || y >= kH2) continue;
+        float d[kH2];
+        load_floats(d, dz + y * kH2);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int ky = r == 1 ? t : t - 1;
+          if (ky < 0 || ky >= kK) continue;
+#pragma unroll
+          for (int j = 0; j < kP1; ++j)
+#pragma unroll
+            for (int kx = 0; kx < kK; ++kx)
+              if (j - kx >= 0 && j - kx < kH2) acc[r][j] = fmaf(d[j - kx], w[ky * kK + kx], acc[r][j]);
+        }
+      }
+    }
+    const long long at = (long long)(i0 + si) * a.c1 * kP1 * kP1 + (ci * kP1 + py0) * kP1;
+    const float* a1 = a.scr + g * a.S + a.o_a1 + at;
+    float* out = a.scr + g * a.S + a.o_dz1 + at;
+#pragma unroll
+    for (int v = 0; v < 2 * kP1 / 4; ++v) {   // the two rows lie one after the other
+      const float4 m = reinterpret_cast<const float4*>(a1)[v];
+      const float* f = &acc[v / 3][4 * (v % 3)];
+      reinterpret_cast<float4*>(out)[v] = make_float4(m.x > 0.f ? f[0] : 0.f, m.y > 0.f ? f[1] : 0.f,
+                                                      m.z > 0.f ? f[2] : 0.f, m.w > 0.f ? f[3] : 0.f);
+    }
+  }
+}
+
+// Per-sample partial sums of conv2's weight and bias gradients: a block per sample, a thread per
+// kernel row (ci, ky) and four output channels, which share each input row.
+constexpr int kW2Threads28 = 256;
+__global__ void __launch_bounds__(kW2Threads28) conv2_wpart28_kernel(const __grid_constant__ ConvArgs a) {
+  gem::pdl_entry();
+  extern __shared__ __align__(16) float sm[];
+  const long long gi = blockIdx.x;
+  const int g = int(gi / a.b), i = int(gi % a.b);
+  const int n_dz2 = a.c2 * kH2 * kH2, n_a1 = a.c1 * kP1 * kP1;
+  float* dzs = sm;                                  // [c2][8][8]
+  float* a1s = dzs + n_dz2;                         // [c1][12][12], channels at kA1Pitch
+  const float* a1 = a.scr + g * a.S + a.o_a1 + (long long)i * n_a1;
+  for (int q = threadIdx.x; q < n_a1 / 4; q += blockDim.x)
+    cp_async16(a1s + q / 36 * kA1Pitch + q % 36 * 4, a1 + 4 * q);
+  rebuild_dz2(dzs, a, g, i);
+  stage_wait();
+  const int per = a.c1 * kK * kK + 1;
+  const int n_rows = a.c1 * kK, n_items = n_rows * ((a.c2 + 3) / 4);
+  float* part = a.scr + g * a.S + a.o_p2 + (long long)i * a.c2 * per;
+  for (int q = threadIdx.x; q < n_items + a.c2; q += blockDim.x) {
+    if (q >= n_items) {
+      const int co = q - n_items;
+      float acc = 0.f;
+#pragma unroll 4
+      for (int y = 0; y < kH2; ++y) {
+        float d[kH2];
+        load_floats(d, dzs + (co * kH2 + y) * kH2);
+#pragma unroll
+        for (int x = 0; x < kH2; ++x) acc += d[x];
+      }
+      part[co * per + per - 1] = acc;
+      continue;
+    }
+    const int row = q % n_rows, ky = row % kK, ci = row / kK, co0 = 4 * (q / n_rows);
+    float acc[4][kK];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int kx = 0; kx < kK; ++kx) acc[c][kx] = 0.f;
+    for (int y = 0; y < kH2; ++y) {
+      float in[kP1];
+      load_floats(in, a1s + ci * kA1Pitch + (ky + y) * kP1);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float d[kH2];
+        load_floats(d, dzs + (min(co0 + c, a.c2 - 1) * kH2 + y) * kH2);
+#pragma unroll
+        for (int x = 0; x < kH2; ++x)
+#pragma unroll
+          for (int kx = 0; kx < kK; ++kx) acc[c][kx] = fmaf(d[x], in[x + kx], acc[c][kx]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (co0 + c < a.c2) {
+#pragma unroll
+        for (int kx = 0; kx < kK; ++kx) part[(co0 + c) * per + (ci * kK + ky) * kK + kx] = acc[c][kx];
+      }
+  }
+}
+
+// Per-sample partial sums of conv1's weight and bias gradients: a block per sample routes the
+// pooled gradient to the windows' maxima in shared memory; then a thread per kernel row (co, ky),
+// and one per bias.
+__global__ void __launch_bounds__(kW1Threads) conv1_wpart28_kernel(const __grid_constant__ ConvArgs a) {
+  gem::pdl_entry();
+  extern __shared__ __align__(16) float sm[];
+  const long long gi = blockIdx.x;
+  const int g = int(gi / a.b), i = int(gi % a.b);
+  float* dzs = sm;                                  // [c1][24][24], channels at kDz1Pitch
+  float* xs = dzs + a.c1 * kDz1Pitch;               // [28][28]
+  stage(xs, a.X + (long long)a.rows[gi] * kH * kH, kH * kH);
+  const uint8_t* k1s = reinterpret_cast<const uint8_t*>(a.scr + g * a.S + a.o_k1) + (long long)i * a.c1 * kP1 * kP1;
+  const float* dp = a.scr + g * a.S + a.o_dz1 + (long long)i * a.c1 * kP1 * kP1;
+  for (int q4 = threadIdx.x; q4 < a.c1 * kP1 * kP1 / 4; q4 += blockDim.x) {   // four windows of a row
+    const float4 v = reinterpret_cast<const float4*>(dp)[q4];
+    const uchar4 am = reinterpret_cast<const uchar4*>(k1s)[q4];
+    const int q = 4 * q4, px = q % kP1, py = q / kP1 % kP1, co = q / (kP1 * kP1);
+    float4* d = reinterpret_cast<float4*>(dzs + co * kDz1Pitch + 2 * py * kH1 + 2 * px);
+    d[0] = make_float4(am.x == 0 ? v.x : 0.f, am.x == 1 ? v.x : 0.f, am.y == 0 ? v.y : 0.f, am.y == 1 ? v.y : 0.f);
+    d[1] = make_float4(am.z == 0 ? v.z : 0.f, am.z == 1 ? v.z : 0.f, am.w == 0 ? v.w : 0.f, am.w == 1 ? v.w : 0.f);
+    d += kH1 / 4;
+    d[0] = make_float4(am.x == 2 ? v.x : 0.f, am.x == 3 ? v.x : 0.f, am.y == 2 ? v.y : 0.f, am.y == 3 ? v.y : 0.f);
+    d[1] = make_float4(am.z == 2 ? v.z : 0.f, am.z == 3 ? v.z : 0.f, am.w == 2 ? v.w : 0.f, am.w == 3 ? v.w : 0.f);
+  }
+  stage_wait();
+  constexpr int per = kK * kK + 1;
+  const int n_rows = a.c1 * kK;
+  float* part = a.scr + g * a.S + a.o_p1 + (long long)i * a.c1 * per;
+  for (int q = threadIdx.x; q < n_rows + a.c1; q += blockDim.x) {
+    if (q >= n_rows) {
+      const int co = q - n_rows;
+      float acc = 0.f;
+#pragma unroll 2
+      for (int y = 0; y < kH1; ++y) {
+        float d[kH1];
+        load_floats(d, dzs + co * kDz1Pitch + y * kH1);
+#pragma unroll
+        for (int x = 0; x < kH1; ++x) acc += d[x];
+      }
+      part[co * per + per - 1] = acc;
+      continue;
+    }
+    const int ky = q % kK, co = q / kK;
+    float acc[kK];
+#pragma unroll
+    for (int kx = 0; kx < kK; ++kx) acc[kx] = 0.f;
+    for (int y = 0; y < kH1; ++y) {
+      float in[kH], d[kH1];
+      load_floats(in, xs + (y + ky) * kH);
+      load_floats(d, dzs + co * kDz1Pitch + y * kH1);
+#pragma unroll
+      for (int x = 0; x < kH1; ++x)
+#pragma unroll
+        for (int kx = 0; kx < kK; ++kx) acc[kx] = fmaf(d[x], in[x + kx], acc[kx]);
+    }
+#pragma unroll
+    for (int kx = 0; kx < kK; ++kx) part[co * per + ky * kK + kx] = acc[kx];
+  }
+}
+
+// Shared memory of the kernels above for c1, c2 channels (floats), in the order conv1_pool,
+// conv2_pool, conv2_back, conv2_wpart, conv1_wpart.
+void smem28(int c1, int c2, long long (&need)[5]) {
+  const long long w2 = (long long)c2 * c1 * kWPitch;
+  need[0] = kH * kH + (long long)c1 * kWPitch;
+  need[1] = w2 + (long long)kPer28 * c1 * kP1 * kP1;
+  need[2] = w2 + (long long)kBackPer28 * c2 * kH2 * kH2;
+  need[3] = (long long)c2 * kH2 * kH2 + c1 * kA1Pitch;
+  need[4] = (long long)c1 * kDz1Pitch + kH * kH;
+}
+
 // Convolution gradients: the partials summed over the minibatch in sample order.
 __global__ void __launch_bounds__(kThreads) conv_finish_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   const int per1 = kK * kK + 1, per2 = a.c1 * kK * kK + 1;
-  const long long n1 = (long long)a.c1 * per1, n2 = (long long)a.c2 * per2;
-  const long long total = (long long)a.G * (n1 + n2);
-  const long long q = blockIdx.x * (long long)kThreads + threadIdx.x;
-  if (q >= total) return;
-  const int g = int(q / (n1 + n2));
-  const long long e = q % (n1 + n2);
+  const int n1 = a.c1 * per1, n2 = a.c2 * per2;
+  const int g = blockIdx.y, e = blockIdx.x * kThreads + threadIdx.x;
+  if (e >= n1 + n2) return;
   float* grad = a.grads + g * a.grad_stride;
   const float* slot = a.scr + g * a.S;
   // kAhead samples' partials in flight, added in sample order
   constexpr int kAhead = 16;
-  auto sum = [&](const float* part, long long ld) {
+  auto sum = [&](const float* part, int ld) {
     float acc = 0.f;
-    for (int i0 = 0; i0 < a.b; i0 += kAhead) {
+    int i0 = 0;
+    for (; i0 + kAhead <= a.b; i0 += kAhead) {
       float v[kAhead];
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u) v[u] = i0 + u < a.b ? part[(i0 + u) * ld] : 0.f;
+      for (int u = 0; u < kAhead; ++u) v[u] = part[(i0 + u) * ld];
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u)
-        if (i0 + u < a.b) acc += v[u];
+      for (int u = 0; u < kAhead; ++u) acc += v[u];
     }
+    for (; i0 < a.b; ++i0) acc += part[i0 * ld];
     return acc;
   };
   if (e < n1) {
-    const int co = int(e / per1), k = int(e % per1);
+    const int co = e / per1, k = e % per1;
     grad[k < per1 - 1 ? a.w1 + co * (per1 - 1) + k : a.b1 + co] = sum(slot + a.o_p1 + co * per1 + k, n1);
   } else {
-    const long long e2 = e - n1;
-    const int co = int(e2 / per2), k = int(e2 % per2);
+    const int e2 = e - n1, co = e2 / per2, k = e2 % per2;
     grad[k < per2 - 1 ? a.w2 + (long long)co * (per2 - 1) + k : a.b2 + co] = sum(slot + a.o_p2 + co * per2 + k, n2);
   }
 }
@@ -514,6 +877,7 @@ struct gem_cnn {
   size_t rows_cap = 0;
   float* pi_rows = nullptr;      // [n][gem stride] scaling factors of a segment's commits
   int smem[5] = {};              // dynamic shared memory of the per-sample kernels (bytes)
+  bool sizes28 = false;          // the kernels of the paper's map sizes
   uint64_t launches = 0;
 };
 
@@ -551,31 +915,35 @@ int cnn_chunk(gem_cnn* N, const int32_t* workers, int G, const int32_t* rows_dev
   const long long n_pool2 = G * b * s.c2 * s.P2 * s.P2;
   int rc;
   const unsigned samples = unsigned(G * b);
-  if (s.H == 28) {
-    gem::launch_pdl(conv1_pool_kernel<28>, samples, kThreads, N->smem[0], st, a);
-    gem::launch_pdl(conv2_pool_kernel<12>, samples, kPool2Threads, N->smem[1], st, a);
+  const unsigned sample_groups = unsigned(G) * unsigned((b + kPer28 - 1) / kPer28);
+  if (N->sizes28) {
+    gem::launch_pdl(conv1_pool28_kernel, samples, kPool1Threads28, N->smem[0], st, a);
+    gem::launch_pdl(conv2_pool28_kernel, sample_groups, kPool2Threads28, N->smem[1], st, a);
   } else {
-    gem::launch_pdl(conv1_pool_kernel<0>, samples, kThreads, N->smem[0], st, a);
-    gem::launch_pdl(conv2_pool_kernel<0>, samples, kPool2Threads, N->smem[1], st, a);
+    gem::launch_pdl(conv1_pool_kernel, samples, kThreads, N->smem[0], st, a);
+    gem::launch_pdl(conv2_pool_kernel, samples, kPool2Threads, N->smem[1], st, a);
   }
   if ((rc = cuda_rc(cudaGetLastError()))) return rc;
   N->launches += 2;
   // the dense head: forward, loss, backward, and the feature gradient
   if ((rc = gem::mlp::mlp_chunk(N->head, workers, G, rows_dev, grads, grad_stride, losses))) return rc;
-  gem::launch_pdl(pool2_back_kernel, blocks_for(n_pool2), kThreads, 0, st, a);
-  if (s.H == 28) {   // the paper's map sizes: loop bounds known at compile time
-    gem::launch_pdl(conv2_back_kernel<8, 12>, samples, kBackThreads, N->smem[2], st, a);
-    gem::launch_pdl(conv2_wpart_kernel<8, 12>, samples, kThreads, N->smem[3], st, a);
-    gem::launch_pdl(conv1_wpart_kernel<24, 28>, samples, kW1Threads, N->smem[4], st, a);
+  if (N->sizes28) {
+    gem::launch_pdl(conv2_back28_kernel, unsigned(G) * unsigned((b + kBackPer28 - 1) / kBackPer28), kBackThreads28,
+                    N->smem[2], st, a);
+    gem::launch_pdl(conv2_wpart28_kernel, samples, kW2Threads28, N->smem[3], st, a);
+    gem::launch_pdl(conv1_wpart28_kernel, samples, kW1Threads, N->smem[4], st, a);
   } else {
-    gem::launch_pdl(conv2_back_kernel<0, 0>, samples, kBackThreads, N->smem[2], st, a);
-    gem::launch_pdl(conv2_wpart_kernel<0, 0>, samples, kThreads, N->smem[3], st, a);
-    gem::launch_pdl(conv1_wpart_kernel<0, 0>, samples, kW1Threads, N->smem[4], st, a);
+    gem::launch_pdl(pool2_back_kernel, blocks_for(n_pool2), kThreads, 0, st, a);
+    gem::launch_pdl(conv2_back_kernel, samples, kBackThreads, N->smem[2], st, a);
+    gem::launch_pdl(conv2_wpart_kernel, samples, kThreads, N->smem[3], st, a);
+    gem::launch_pdl(conv1_wpart_kernel, samples, kW1Threads, N->smem[4], st, a);
+    N->launches += 1;
   }
-  gem::launch_pdl(conv_finish_kernel, blocks_for(G * ((long long)s.c1 * (kK * kK + 1) +
-                                       (long long)s.c2 * (s.c1 * kK * kK + 1))), kThreads, 0, st, a);
+  gem::launch_pdl(conv_finish_kernel, dim3(blocks_for((long long)s.c1 * (kK * kK + 1) +
+                                                      (long long)s.c2 * (s.c1 * kK * kK + 1)), unsigned(G)),
+                  kThreads, 0, st, a);
   if ((rc = cuda_rc(cudaGetLastError()))) return rc;
-  N->launches += 5;
+  N->launches += 4;
   return GEM_OK;
 }
 
@@ -648,12 +1016,6 @@ int gem_cnn_create(gem_t* g, const int32_t* shape, int batch, gem_cnn_t** out) {
         f * (s.c2 * s.H2 * (s.H2 + 1) + (long long)s.c2 * s.c1 * kK * kK + s.c1 * s.P1 * s.P1),  // conv2_back
         f * (s.c2 * s.H2 * s.H2 + s.c1 * s.P1 * s.P1),                              // conv2_wpart
         f * (s.c1 * s.H1 * s.H1 + s.H * s.H)};                                      // conv1_wpart
-    // per kernel, the generic instantiation and the one for the paper's map sizes
-    const void* fn[5][2] = {{(const void*)conv1_pool_kernel<0>, (const void*)conv1_pool_kernel<28>},
-                            {(const void*)conv2_pool_kernel<0>, (const void*)conv2_pool_kernel<12>},
-                            {(const void*)conv2_back_kernel<0, 0>, (const void*)conv2_back_kernel<8, 12>},
-                            {(const void*)conv2_wpart_kernel<0, 0>, (const void*)conv2_wpart_kernel<8, 12>},
-                            {(const void*)conv1_wpart_kernel<0, 0>, (const void*)conv1_wpart_kernel<24, 28>}};
     for (int k = 0; k < 5; ++k) {
       if (need[k] > kMaxSampleSmem) {   // a sample's maps and weights must fit on chip
         gem::mlp::mlp_free(N->head);
@@ -661,12 +1023,24 @@ int gem_cnn_create(gem_t* g, const int32_t* shape, int batch, gem_cnn_t** out) {
         return GEM_EINVAL;
       }
       N->smem[k] = int(need[k]);
-      bool ok = true;
-      for (int v = 0; v < 2 && need[k] > 48 * 1024; ++v)
-        if (fn[k][v] && cudaFuncSetAttribute(fn[k][v], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(need[k])) != cudaSuccess)
-          ok = false;
-      if (!ok) {
+    }
+    // the kernels for the paper's map sizes, while their staging (two samples, padded weights) fits
+    long long need28[5];
+    smem28(s.c1, s.c2, need28);
+    N->sizes28 = s.H == kH;
+    for (int k = 0; k < 5; ++k) N->sizes28 = N->sizes28 && f * need28[k] <= kMaxSmem28;
+    const void* fn[2][5] = {{(const void*)conv1_pool_kernel, (const void*)conv2_pool_kernel,
+                             (const void*)conv2_back_kernel, (const void*)conv2_wpart_kernel,
+                             (const void*)conv1_wpart_kernel},
+                            {(const void*)conv1_pool28_kernel, (const void*)conv2_pool28_kernel,
+                             (const void*)conv2_back28_kernel, (const void*)conv2_wpart28_kernel,
+                             (const void*)conv1_wpart28_kernel}};
+    for (int k = 0; k < 5; ++k) {
+      if (N->sizes28) N->smem[k] = int(f * need28[k]);
+      // the limit, not this network's need: the attribute is the kernel's, for every network
+      if (N->smem[k] > 48 * 1024 &&
+          cudaFuncSetAttribute(fn[N->sizes28 ? 1 : 0][k], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(N->sizes28 ? kMaxSmem28 : kMaxSampleSmem)) != cudaSuccess) {
         cudaGetLastError();
         gem::mlp::mlp_free(N->head);
         delete N;

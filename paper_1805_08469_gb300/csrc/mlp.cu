@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(256)
 bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
                  long long slot_stride, float* grad, long long grad_stride) {
   gem::pdl_entry();
-  constexpr int kAhead = 16;
+  constexpr int kAhead = 8;
   __shared__ float part[8][33];
   __shared__ float row_loss[kMaxBatch];
   const int g = blockIdx.y;
@@ -1232,14 +1232,16 @@ bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
     o = q - a.first[l];
     const float* D = delta + g * slot_stride + a.delta_off[l] + o;
     const long long ld = a.width[l];
-    for (int r0 = y; r0 < a.b; r0 += 8 * kAhead) {   // kAhead rows in flight, added in order
+    int r = y;
+    for (; r + 8 * (kAhead - 1) < a.b; r += 8 * kAhead) {   // kAhead rows in flight, added in order
       float v[kAhead];
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u) v[u] = r0 + 8 * u < a.b ? D[(r0 + 8 * u) * ld] : 0.f;
+      for (int u = 0; u < kAhead; ++u) v[u] = D[(r + 8 * u) * ld];
 #pragma unroll
-      for (int u = 0; u < kAhead; ++u)
-        if (r0 + 8 * u < a.b) s += v[u];
+      for (int u = 0; u < kAhead; ++u) s += v[u];
     }
+#pragma unroll 4
+    for (; r < a.b; r += 8) s += D[r * ld];
   }
   part[y][x] = s;
   __syncthreads();
