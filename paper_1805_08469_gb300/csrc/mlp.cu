@@ -132,6 +132,17 @@ __device__ __forceinline__ uint32_t tf32_bits(float x) {
   return r;
 }
 
+// Two fp32 values in one register pair, and the packed FMA on pairs: each component is rounded
+// as fmaf rounds it.
+__device__ __forceinline__ unsigned long long pair_of(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void fma_pair(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
 // Four consecutive elements (outer, inner .. inner + 3) of a row-major view with leading
 // dimension ld: one 16-byte load when the rows are 16-byte aligned (vec) and the quad lies
 // inside the operand, else element by element; zeros outside.  TF32: each value rounded.
@@ -166,8 +177,14 @@ __device__ __forceinline__ float4 stage_quad(const float* base, long long ld, bo
 // TBM x 64 tile per block of 2 TBM threads; thread (tx, ty) = (tid % 16, tid / 16) owns
 // rows 8 ty .. 8 ty + 7 and columns 4 tx .. 4 tx + 3.  Both tiles are kept m- (or n-) contiguous
 // in shared memory, double-buffered, so one k-step is three 128-bit shared loads and 32
-// FMAs.  The next k-tile is read from global memory into registers while the current one
-// is multiplied; global reads are coalesced along whichever index is contiguous.
+// FMAs: 16 packed ones, on pairs of rows as they lie in shared memory (the scalar FMA issues
+// 112 per cycle and SM at most, held up by its operand reads; the packed one passed 180 with
+// two warps per scheduler).  The next k-tile is read from global memory into registers while
+// the current one is multiplied; global reads are coalesced along whichever index is
+// contiguous, and a thread's four columns of a row are stored as one 16-byte word.
+// What bounds it now is the shared-memory reads (two thirds of their rate with 7 to 11 warps per
+// SM).  784-1000-1000-10, n = 30 in fp32, 48 commits: 2,249 us with scalar FMAs, 2,134 packed,
+// 2,104 with the wide stores.
 template <int TBM, bool A_KMAJOR, bool B_KMAJOR, int EPI, bool TF32>
 __global__ void __launch_bounds__(2 * TBM)
 gemm_grouped_kernel(const __grid_constant__ GemmArgs p) {
@@ -238,11 +255,12 @@ gemm_grouped_kernel(const __grid_constant__ GemmArgs p) {
     }
   };
 
-  float acc[8][4];
+  // acc[i][j]: rows 2 i and 2 i + 1 of column j
+  unsigned long long acc[4][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
 
   load(kbeg);
   store(0);
@@ -253,15 +271,16 @@ gemm_grouped_kernel(const __grid_constant__ GemmArgs p) {
     if (more) load(k0 + BK);
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 8 + 4]);
+      const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(&As[buf][k][ty * 8]);
+      const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(&As[buf][k][ty * 8 + 4]);
       const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+      const unsigned long long a[4] = {a0.x, a0.y, a1.x, a1.y};
+      const unsigned long long b[4] = {pair_of(b4.x, b4.x), pair_of(b4.y, b4.y), pair_of(b4.z, b4.z),
+                                       pair_of(b4.w, b4.w)};
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) fma_pair(acc[i][j], a[i], b[j]);
     }
     if (more) {
       store(buf ^ 1);   // the other buffer was last read before the previous barrier
@@ -270,23 +289,44 @@ gemm_grouped_kernel(const __grid_constant__ GemmArgs p) {
     }
   }
 
+  float out[8][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(out[2 * i][j]), "=f"(out[2 * i + 1][j]) : "l"(acc[i][j]));
+  // a thread's four columns of a row are stored as one 16-byte word where the row allows it
+  const int n = n0 + tx * 4;
+  auto store4 = [&](float* row, const float (&v)[4], bool vec) {
+    if (vec && n + 3 < N) {
+      *reinterpret_cast<float4*>(row + n) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (n + j < N) row[n + j] = v[j];
+    }
+  };
+  auto aligned = [](const float* base, long long ld) {
+    return (reinterpret_cast<uintptr_t>(base) & 15u) == 0 && (ld & 3) == 0;
+  };
   if (split > 1) {  // raw partial sums; splitk_reduce_kernel applies the epilogue
     float* W = p.ws + (long long)blockIdx.z * M * N;
+    const bool vec = aligned(W, N);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int m = m0 + ty * 8 + i;
-      if (m >= M) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int n = n0 + tx * 4 + j;
-        if (n < N) W[(long long)m * N + n] = acc[i][j];
-      }
+      if (m < M) store4(W + (long long)m * N, out[i], vec);
     }
     return;
   }
   float* C = p.C + (long long)g * p.c_group_stride;
-  const float* bias = (EPI == kBias || EPI == kBiasRelu)
-                          ? p.bias + (long long)p.workers[g] * p.bias_group_stride : nullptr;
+  const bool vec = aligned(C, p.ldc);
+  float bias[4] = {0.f, 0.f, 0.f, 0.f};
+  if (EPI == kBias || EPI == kBiasRelu) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (n + j < N) bias[j] = p.bias[(long long)p.workers[g] * p.bias_group_stride + n + j];
+  }
   const float* mask = EPI == kMask ? p.mask + (long long)g * p.mask_group_stride : nullptr;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -294,14 +334,12 @@ gemm_grouped_kernel(const __grid_constant__ GemmArgs p) {
     if (m >= M) continue;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      float v = acc[i][j];
-      if (EPI == kBias) v = v + bias[n];
-      if (EPI == kBiasRelu) v = fmaxf(v + bias[n], 0.f);
-      if (EPI == kMask) v = mask[m * p.ldmask + n] > 0.f ? v : 0.f;
-      C[m * p.ldc + n] = v;
+      float& v = out[i][j];
+      if (EPI == kBias) v = v + bias[j];
+      if (EPI == kBiasRelu) v = fmaxf(v + bias[j], 0.f);
+      if (EPI == kMask && n + j < N) v = mask[m * p.ldmask + n + j] > 0.f ? v : 0.f;
     }
+    store4(C + m * p.ldc, out[i], vec);
   }
 }
 
