@@ -417,45 +417,48 @@ __device__ __forceinline__ void simt_stage(float* dst, const float* src, long lo
   }
 }
 
-template <int BM, bool A_KMAJOR, bool B_KMAJOR, int EPI, bool TF32>
-__global__ void __launch_bounds__(kSimtThreads, 4)
-gemm_simt_kernel(const __grid_constant__ GemmArgs p) {
-  gem::pdl_entry();
+// One operand of one group: base, leading dimension, and (or null) its storage rows in order.
+struct SimtOperand {
+  const float* base;
+  long long ld;
+  const int32_t* rows;
+  int n_rows;
+};
+
+__device__ __forceinline__ SimtOperand simt_operand(const Operand& o, const int* workers, int g) {
+  return SimtOperand{o.base + (o.by_worker ? (long long)workers[g] : (long long)g) * o.group_stride, o.ld,
+                     o.rows ? o.rows + (long long)g * o.rows_per_group : nullptr, o.rows_per_group};
+}
+
+// The sums of a block's tile (rows m0.., columns n0.. of M x N) over k in [kbeg, kend).
+template <int BM, bool A_KMAJOR, bool B_KMAJOR, bool TF32>
+__device__ __forceinline__ void simt_tile(const SimtOperand& A, const SimtOperand& B, int M, int N, int m0, int n0,
+                                          int kbeg, int kend, float* smem, int32_t* row_idx,
+                                          float (&acc)[SimtTile<BM>::TM][SimtTile<BM>::TN]) {
   using Tile = SimtTile<BM>;
   constexpr int TM = Tile::TM, TN = Tile::TN, TX = Tile::TX, TY = Tile::TY;
   constexpr int kA = simt_tile_floats(BM, A_KMAJOR), kStage = kA + simt_tile_floats(BN, B_KMAJOR);
-  extern __shared__ __align__(16) float simt_smem[];
-  __shared__ int32_t row_idx[kMaxBatch];
-  const int split = p.ksplit;
-  const int g = blockIdx.z / split, sk = blockIdx.z - g * split;
-  const int kbeg = sk * p.kchunk, kend = min(p.K, kbeg + p.kchunk);
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-  const float* A = p.A.base + (p.A.by_worker ? (long long)p.workers[g] : (long long)g) * p.A.group_stride;
-  const float* B = p.B.base + (p.B.by_worker ? (long long)p.workers[g] : (long long)g) * p.B.group_stride;
-  const int M = p.M, N = p.N;
-  const bool a_vec = (reinterpret_cast<uintptr_t>(A) & 15u) == 0 && (p.A.ld & 3) == 0;
-  const bool b_vec = (reinterpret_cast<uintptr_t>(B) & 15u) == 0 && (p.B.ld & 3) == 0;
-  const int32_t* idx = p.A.rows ? p.A.rows : p.B.rows;   // at most one operand reads by index
+  const bool a_vec = (reinterpret_cast<uintptr_t>(A.base) & 15u) == 0 && (A.ld & 3) == 0;
+  const bool b_vec = (reinterpret_cast<uintptr_t>(B.base) & 15u) == 0 && (B.ld & 3) == 0;
+  const int32_t* idx = A.rows ? A.rows : B.rows;   // at most one operand reads by index
   if (idx) {
-    const int n_rows = p.A.rows ? p.A.rows_per_group : p.B.rows_per_group;
-    for (int i = tid; i < n_rows; i += kSimtThreads) row_idx[i] = idx[(long long)g * n_rows + i];
+    const int n_rows = A.rows ? A.n_rows : B.n_rows;
+    for (int i = tid; i < n_rows; i += kSimtThreads) row_idx[i] = idx[i];
     __syncthreads();
   }
-  const int32_t* a_idx = p.A.rows ? row_idx : nullptr;
-  const int32_t* b_idx = p.B.rows ? row_idx : nullptr;
-
+  const int32_t* a_idx = A.rows ? row_idx : nullptr;
+  const int32_t* b_idx = B.rows ? row_idx : nullptr;
   const int nkt = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
   auto issue = [&](int kt) {
     if (kt < nkt) {
-      float* st = simt_smem + kt % kSimtStages * kStage;
+      float* st = smem + kt % kSimtStages * kStage;
       const int k0 = kbeg + kt * BK;
-      simt_stage<BM, A_KMAJOR>(st, A, p.A.ld, a_idx, a_vec, m0, M, k0, kend);
-      simt_stage<BN, B_KMAJOR>(st + kA, B, p.B.ld, b_idx, b_vec, n0, N, k0, kend);
+      simt_stage<BM, A_KMAJOR>(st, A.base, A.ld, a_idx, a_vec, m0, M, k0, kend);
+      simt_stage<BN, B_KMAJOR>(st + kA, B.base, B.ld, b_idx, b_vec, n0, N, k0, kend);
     }
     cp_async_commit();
   };
-  float acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -469,7 +472,7 @@ gemm_simt_kernel(const __grid_constant__ GemmArgs p) {
     cp_async_wait<kSimtStages - 2>();
     __syncthreads();   // everyone's copies of k-tile kt have landed; k-tile kt - 1 has been read
     issue(kt + kSimtStages - 1);
-    const float* As = simt_smem + kt % kSimtStages * kStage;
+    const float* As = smem + kt % kSimtStages * kStage;
     const float* Bs = As + kA;
 #pragma unroll
     for (int k = 0; k < BK; k += 4) {
@@ -505,6 +508,24 @@ gemm_simt_kernel(const __grid_constant__ GemmArgs p) {
           for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i][q], b[j][q], acc[i][j]);
     }
   }
+}
+
+template <int BM, bool A_KMAJOR, bool B_KMAJOR, int EPI, bool TF32>
+__global__ void __launch_bounds__(kSimtThreads, 4)
+gemm_simt_kernel(const __grid_constant__ GemmArgs p) {
+  gem::pdl_entry();
+  using Tile = SimtTile<BM>;
+  constexpr int TM = Tile::TM, TN = Tile::TN, TX = Tile::TX, TY = Tile::TY;
+  extern __shared__ __align__(16) float simt_smem[];
+  __shared__ int32_t row_idx[kMaxBatch];
+  const int split = p.ksplit;
+  const int g = blockIdx.z / split, sk = blockIdx.z - g * split;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  const int M = p.M, N = p.N;
+  float acc[TM][TN];
+  simt_tile<BM, A_KMAJOR, B_KMAJOR, TF32>(simt_operand(p.A, p.workers, g), simt_operand(p.B, p.workers, g), M, N, m0,
+                                          n0, sk * p.kchunk, min(p.K, (sk + 1) * p.kchunk), simt_smem, row_idx, acc);
 
   // tile coordinates of this thread's outputs
   auto row_of = [&](int i) { return A_KMAJOR ? ty + TY * i : (i / 4) * (4 * TY) + 4 * ty + i % 4; };
@@ -544,9 +565,9 @@ gemm_simt_kernel(const __grid_constant__ GemmArgs p) {
   cluster.sync();
   const int rows = min(BM, M - m0), per = (rows + split - 1) / split;
   const int r_end = min(rows, (sk + 1) * per);
-  const int c = tid % BN, n = n0 + c;
+  const int c = threadIdx.x % BN, n = n0 + c;
   if (n < N) {
-    for (int r = sk * per + tid / BN; r < r_end; r += kSimtThreads / BN) {
+    for (int r = sk * per + threadIdx.x / BN; r < r_end; r += kSimtThreads / BN) {
       float v = 0.f;
       for (int q = 0; q < split; ++q) v += cluster.map_shared_rank(simt_smem, q)[r * kPartPitch + c];
       finish(v, m0 + r, n);
@@ -1245,54 +1266,130 @@ struct BiasGradArgs {
   int first[kMaxLayers + 1];        // prefix sums of width
 };
 
-// db_l[o] = sum over the batch of D_{l+1}[r][o], every layer in one launch.
-// Block of 32 x 8 threads: lane x owns output q = 32 blockIdx.x + x; warp y sums rows
-// r = y, y + 8, ... in order, and lane x of warp 0 adds the 8 warp sums in order.  When
-// the logits kernel computed the loss (losses set), thread 0 of block (0, g) also adds
-// group g's row losses in row order and divides by b.
-__global__ void __launch_bounds__(256)
-bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
-                 long long slot_stride, float* grad, long long grad_stride) {
-  gem::pdl_entry();
+// db_l[o] = sum over the batch of D_{l+1}[r][o] for the 32 outputs q of block `block` of group g
+// (every layer's outputs in turn), by T = 128 or 256 threads: lane x owns output q = 32 block +
+// x; partial y = 0..7 sums rows r = y, y + 8, ... in order (warp y, and warp y - 4 too with 128
+// threads), and warp 0 adds the 8 partials in order.  When the logits kernel computed the loss
+// (losses set), thread 0 of block 0 also adds the group's row losses in row order and divides
+// by b.  part: 8 x 33 floats of shared memory, row_loss: kMaxBatch.
+template <int T>
+__device__ __forceinline__ void bias_grad_block(const BiasGradArgs& a, const float* delta, long long slot_stride,
+                                                float* grad, long long grad_stride, int block, int g, float* part,
+                                                float* row_loss) {
   constexpr int kAhead = 8;
-  __shared__ float part[8][33];
-  __shared__ float row_loss[kMaxBatch];
-  const int g = blockIdx.y;
-  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-  const int q = blockIdx.x * 32 + x;
-  const bool sums_loss = a.losses && blockIdx.x == 0;
+  const int x = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int q = block * 32 + x;
+  const bool sums_loss = a.losses && block == 0;
   if (sums_loss)
-    for (int r = threadIdx.x; r < a.b; r += 256) row_loss[r] = delta[g * slot_stride + a.row_loss_off + r];
-  float s = 0.f;
+    for (int r = threadIdx.x; r < a.b; r += T) row_loss[r] = delta[g * slot_stride + a.row_loss_off + r];
   int l = 0, o = 0;
   if (q < a.first[a.n_layers]) {
     while (q >= a.first[l + 1]) ++l;
     o = q - a.first[l];
-    const float* D = delta + g * slot_stride + a.delta_off[l] + o;
-    const long long ld = a.width[l];
-    int r = y;
-    for (; r + 8 * (kAhead - 1) < a.b; r += 8 * kAhead) {   // kAhead rows in flight, added in order
-      float v[kAhead];
-#pragma unroll
-      for (int u = 0; u < kAhead; ++u) v[u] = D[(r + 8 * u) * ld];
-#pragma unroll
-      for (int u = 0; u < kAhead; ++u) s += v[u];
-    }
-#pragma unroll 4
-    for (; r < a.b; r += 8) s += D[r * ld];
   }
-  part[y][x] = s;
+  for (int y = warp; y < 8; y += T / 32) {
+    float s = 0.f;
+    if (q < a.first[a.n_layers]) {
+      const float* D = delta + g * slot_stride + a.delta_off[l] + o;
+      const long long ld = a.width[l];
+      int r = y;
+      for (; r + 8 * (kAhead - 1) < a.b; r += 8 * kAhead) {   // kAhead rows in flight, added in order
+        float v[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) v[u] = D[(r + 8 * u) * ld];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) s += v[u];
+      }
+#pragma unroll 4
+      for (; r < a.b; r += 8) s += D[r * ld];
+    }
+    part[y * 33 + x] = s;
+  }
   __syncthreads();
-  if (y == 0 && q < a.first[a.n_layers]) {
+  if (warp == 0 && q < a.first[a.n_layers]) {
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) t += part[w][x];
+    for (int y = 0; y < 8; ++y) t += part[y * 33 + x];
     grad[g * grad_stride + a.grad_off[l] + o] = t;
   }
   if (sums_loss && threadIdx.x == 0) {   // the minibatch loss, rows in order
     float t = 0.f;
     for (int r = 0; r < a.b; ++r) t += row_loss[r];
     a.losses[g] = t / float(a.b);
+  }
+}
+
+__global__ void __launch_bounds__(256)
+bias_grad_kernel(const __grid_constant__ BiasGradArgs a, const float* delta,
+                 long long slot_stride, float* grad, long long grad_stride) {
+  gem::pdl_entry();
+  __shared__ float part[8 * 33];
+  __shared__ float row_loss[kMaxBatch];
+  bias_grad_block<256>(a, delta, slot_stride, grad, grad_stride, blockIdx.x, blockIdx.y, part, row_loss);
+}
+
+// Every weight gradient dW_l = D_{l+1}^T A_l of a network whose products are small, with the bias
+// gradients and the minibatch loss, in one launch after the delta chain: the tiles of the
+// layers follow each other in blockIdx.x, then the blocks of 32 bias gradients; group g is
+// blockIdx.y.  Launched one by one on the second stream these took an event each way per
+// layer and left the chain to wait for the last of them.
+// Measured: 784-64-10, n = 4, 64 commits 886 -> 668 us; the MNIST network, n = 100, 847 -> 827 us.
+struct WeightGradArgs {
+  int n_layers, b;
+  const float* X;                   // the data set when the first layer reads it in place, else null
+  const int32_t* batch_rows;        // [groups][b]
+  const float* scratch;             // slot g at scratch + g * slot_stride
+  long long slot_stride;
+  long long off_delta[kMaxLayers];  // D_{l+1} in the slot
+  long long off_act[kMaxLayers];    // A_l in the slot
+  long long w_off[kMaxLayers];      // dW_l in the gradient
+  int dims[kMaxLayers + 1];
+  int first[kMaxLayers + 1];        // first tile of layer l; the bias blocks follow the last
+  float* grads;
+  long long grad_stride;
+};
+
+__global__ void __launch_bounds__(kSimtThreads, 4)
+weight_grad_kernel(const __grid_constant__ WeightGradArgs w, const __grid_constant__ BiasGradArgs bias) {
+  gem::pdl_entry();
+  constexpr int BM = 32;
+  using Tile = SimtTile<BM>;
+  extern __shared__ __align__(16) float simt_smem[];
+  __shared__ int32_t row_idx[kMaxBatch];
+  const int g = blockIdx.y;
+  const int t = blockIdx.x;
+  if (t >= w.first[w.n_layers]) {
+    bias_grad_block<kSimtThreads>(bias, w.scratch, w.slot_stride, w.grads, w.grad_stride,
+                                  t - w.first[w.n_layers], g, simt_smem, reinterpret_cast<float*>(row_idx));
+    return;
+  }
+  int l = 0;
+  while (t >= w.first[l + 1]) ++l;
+  const int M = w.dims[l + 1], N = w.dims[l];
+  const int nt = (N + BN - 1) / BN, mt = (t - w.first[l]) / nt;
+  const int m0 = mt * BM, n0 = (t - w.first[l] - mt * nt) * BN;
+  const float* slot = w.scratch + g * w.slot_stride;
+  const SimtOperand A = {slot + w.off_delta[l], M, nullptr, 0};
+  const SimtOperand B = l == 0 && w.X ? SimtOperand{w.X, N, w.batch_rows + (long long)g * w.b, w.b}
+                                      : SimtOperand{slot + w.off_act[l], N, nullptr, 0};
+  float acc[Tile::TM][Tile::TN];
+  simt_tile<BM, false, false, false>(A, B, M, N, m0, n0, 0, w.b, simt_smem, row_idx, acc);
+  const int tx = threadIdx.x % Tile::TX, ty = threadIdx.x / Tile::TX;
+  float* C = w.grads + g * w.grad_stride + w.w_off[l];
+  const int n = n0 + 4 * tx;
+  const bool vec = (reinterpret_cast<uintptr_t>(C) & 15u) == 0 && (N & 3) == 0;
+#pragma unroll
+  for (int i = 0; i < Tile::TM; ++i) {
+    const int m = m0 + 4 * ty + i;
+    if (m >= M) continue;
+    float* row = C + (long long)m * N;
+    if (vec && n + 3 < N) {
+      *reinterpret_cast<float4*>(row + n) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < Tile::TN; ++j)
+        if (n + j < N) row[n + j] = acc[i][j];
+    }
   }
 }
 
@@ -1665,50 +1762,104 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
     M->launches++;
   }
 
-  // backward.  The weight-gradient products go to the side stream when there is one: each
-  // waits for its delta D_{l+1} (event recorded on the main stream) and runs next to the
-  // input-gradient chain; they use no split-K workspace, which belongs to the main stream.
+  BiasGradArgs ba;
+  std::memset(&ba, 0, sizeof(ba));
+  ba.n_layers = L;
+  ba.b = b;
+  ba.row_loss_off = M->off_row_loss;
+  ba.losses = fused_loss ? losses : nullptr;
+  ba.first[0] = 0;
+  for (int l = 0; l < L; ++l) {
+    ba.grad_off[l] = M->b_off[l];
+    ba.delta_off[l] = M->off_delta[l + 1];
+    ba.width[l] = M->dims[l + 1];
+    ba.first[l + 1] = ba.first[l] + M->dims[l + 1];
+  }
+  // Small networks: the weight and bias gradients in one launch, once the deltas are known; on
+  // the main stream, or on the side stream next to the input gradient and what the caller
+  // does with it.
+  bool merged = !tf32;
+  for (int l = 0; l < L; ++l) merged = merged && small_product(M->dims[l + 1], M->dims[l], b, G);
+  const bool aside = merged && two_streams && M->input_grad;
+  auto weight_grads = [&]() -> int {
+    WeightGradArgs wa;
+    std::memset(&wa, 0, sizeof(wa));
+    wa.n_layers = L;
+    wa.b = b;
+    wa.X = in_place ? M->X : nullptr;
+    wa.batch_rows = batch_rows;
+    wa.scratch = scr;
+    wa.slot_stride = S;
+    for (int l = 0; l < L; ++l) {
+      wa.off_delta[l] = M->off_delta[l + 1];
+      wa.off_act[l] = l == 0 ? M->off_x : M->off_act[l];
+      wa.w_off[l] = M->w_off[l];
+      wa.first[l + 1] = wa.first[l] + (M->dims[l + 1] + 31) / 32 * ((M->dims[l] + BN - 1) / BN);
+    }
+    for (int l = 0; l <= L; ++l) wa.dims[l] = M->dims[l];
+    wa.grads = grads;
+    wa.grad_stride = grad_stride;
+    constexpr int bytes = 4 * simt_smem_floats(32, false, false);
+    static_assert(bytes <= 40 * 1024, "within the default limit");
+    if (aside) {
+      int r = cuda_rc(cudaEventRecord(M->ev_delta[1], st));
+      if (r == GEM_OK) r = cuda_rc(cudaStreamWaitEvent(wst, M->ev_delta[1], 0));
+      if (r) return r;
+    }
+    gem::launch_pdl(weight_grad_kernel, dim3(unsigned(wa.first[L] + (ba.first[L] + 31) / 32), unsigned(G)),
+                    kSimtThreads, size_t(bytes), aside ? wst : st, wa, ba);
+    M->launches++;
+    return cuda_rc(cudaGetLastError());
+  };
+
+  // backward.  The weight-gradient products of larger networks go to the side stream when there
+  // is one: each waits for its delta D_{l+1} (event recorded on the main stream) and runs next
+  // to the input-gradient chain; they use no split-K workspace, which belongs to the main stream.
   for (int l = L - 1; l >= 0; --l) {
     const int din = M->dims[l], dout = M->dims[l + 1];
-    if (two_streams) {
-      if ((rc = cuda_rc(cudaEventRecord(M->ev_delta[l + 1], st)))) return rc;
-      if ((rc = cuda_rc(cudaStreamWaitEvent(wst, M->ev_delta[l + 1], 0)))) return rc;
-    }
-    // dW_l = D_{l+1}^T A_l: (m = o, k = r) from D [b x dout], (k = r, n = j) from A [b x din],
-    // or from the transposes D^T [dout x b] and A^T [din x b], both K-major and TF32
-    GemmArgs w = a;
-    w.M = dout; w.N = din; w.K = b;
-    w.round_c = 0;
-    w.C = grads + M->w_off[l];
-    w.c_group_stride = grad_stride;
-    w.ldc = din;
-    if (two_streams) {
-      w.ws = nullptr;
-      w.can_split = 0;
-    }
-    w.bias = nullptr;
-    w.mask = nullptr;
-    cudaError_t ew;
-    if (t_dw(l)) {
-      // D_{l+1}^T, on the weight-gradient stream (the input-gradient chain goes on)
-      if ((rc = transpose(wst, scr + M->off_delta[l + 1], S, false, scr + M->off_deltaT[l + 1], b, dout)))
-        return rc;
-      w.A = Operand{scr + M->off_deltaT[l + 1], S, b, 0, nullptr, 0};
-      w.B = Operand{scr + M->off_actT[l], S, b, 0, nullptr, 0};
-      w.a_rounded = 1;
-      w.b_rounded = 1;
-      set_extents(w, G);
-      ew = launch_gemm<true, true, kStore>(w, G, tf32, wst);
+    if (merged) {
+      if (l == 0 && (rc = weight_grads())) return rc;
     } else {
-      w.A = Operand{scr + M->off_delta[l + 1], S, dout, 0, nullptr, 0};
-      w.B = l == 0 && in_place ? Operand{M->X, 0, din, 0, batch_rows, b} : Operand{act(l), S, din, 0, nullptr, 0};
-      w.a_rounded = 0;
-      w.b_rounded = 0;
-      set_extents(w, G);
-      ew = launch_gemm<false, false, kStore>(w, G, tf32, wst);
+      if (two_streams) {
+        if ((rc = cuda_rc(cudaEventRecord(M->ev_delta[l + 1], st)))) return rc;
+        if ((rc = cuda_rc(cudaStreamWaitEvent(wst, M->ev_delta[l + 1], 0)))) return rc;
+      }
+      // dW_l = D_{l+1}^T A_l: (m = o, k = r) from D [b x dout], (k = r, n = j) from A [b x din],
+      // or from the transposes D^T [dout x b] and A^T [din x b], both K-major and TF32
+      GemmArgs w = a;
+      w.M = dout; w.N = din; w.K = b;
+      w.round_c = 0;
+      w.C = grads + M->w_off[l];
+      w.c_group_stride = grad_stride;
+      w.ldc = din;
+      if (two_streams) {
+        w.ws = nullptr;
+        w.can_split = 0;
+      }
+      w.bias = nullptr;
+      w.mask = nullptr;
+      cudaError_t ew;
+      if (t_dw(l)) {
+        // D_{l+1}^T, on the weight-gradient stream (the input-gradient chain goes on)
+        if ((rc = transpose(wst, scr + M->off_delta[l + 1], S, false, scr + M->off_deltaT[l + 1], b, dout)))
+          return rc;
+        w.A = Operand{scr + M->off_deltaT[l + 1], S, b, 0, nullptr, 0};
+        w.B = Operand{scr + M->off_actT[l], S, b, 0, nullptr, 0};
+        w.a_rounded = 1;
+        w.b_rounded = 1;
+        set_extents(w, G);
+        ew = launch_gemm<true, true, kStore>(w, G, tf32, wst);
+      } else {
+        w.A = Operand{scr + M->off_delta[l + 1], S, dout, 0, nullptr, 0};
+        w.B = l == 0 && in_place ? Operand{M->X, 0, din, 0, batch_rows, b} : Operand{act(l), S, din, 0, nullptr, 0};
+        w.a_rounded = 0;
+        w.b_rounded = 0;
+        set_extents(w, G);
+        ew = launch_gemm<false, false, kStore>(w, G, tf32, wst);
+      }
+      if ((rc = cuda_rc(ew))) return rc;
+      M->launches++;
     }
-    if ((rc = cuda_rc(ew))) return rc;
-    M->launches++;
     if (l == 0) {
       if (!M->input_grad) break;
       // D_0 = D_1 W_0, the gradient with respect to the input rows (no activation here)
@@ -1743,24 +1894,13 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
     if ((rc = cuda_rc(launch_gemm<true, false, kMask>(a, G, tf32, st)))) return rc;
     M->launches++;
   }
-  BiasGradArgs ba;
-  std::memset(&ba, 0, sizeof(ba));
-  ba.n_layers = L;
-  ba.b = b;
-  ba.row_loss_off = M->off_row_loss;
-  ba.losses = fused_loss ? losses : nullptr;
-  ba.first[0] = 0;
-  for (int l = 0; l < L; ++l) {
-    ba.grad_off[l] = M->b_off[l];
-    ba.delta_off[l] = M->off_delta[l + 1];
-    ba.width[l] = M->dims[l + 1];
-    ba.first[l + 1] = ba.first[l] + M->dims[l + 1];
+  if (!merged) {
+    gem::launch_pdl(bias_grad_kernel, dim3((ba.first[L] + 31) / 32, G), 256, 0, st, ba, scr, S, grads,
+                    grad_stride);
+    if ((rc = cuda_rc(cudaGetLastError()))) return rc;
+    M->launches++;
   }
-  gem::launch_pdl(bias_grad_kernel, dim3((ba.first[L] + 31) / 32, G), 256, 0, st, ba, scr, S, grads,
-                                                                      grad_stride);
-  if ((rc = cuda_rc(cudaGetLastError()))) return rc;
-  M->launches++;
-  if (two_streams) {   // the gradients are complete once the side stream is
+  if (two_streams && (!merged || aside)) {   // the gradients are complete once the side stream is
     if ((rc = cuda_rc(cudaEventRecord(M->ev_side, wst)))) return rc;
     if ((rc = cuda_rc(cudaStreamWaitEvent(st, M->ev_side, 0)))) return rc;
   }
