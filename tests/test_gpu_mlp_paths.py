@@ -4,9 +4,11 @@ The gradients are compared with the oracle at the bars of test_gpu_mlp.  The bar
 cases is the 1e-5 of that file: sums of K products in fp32, one rounding of 6e-8 each, grow
 as sqrt(K) at random, 2e-6 for the K = 1,000 of the longest.
 """
+import numpy as np
 import pytest
+import torch
 
-from paper_1805_08469_gb300 import sim
+from paper_1805_08469_gb300 import gem, sim, synth, synth_gpu
 
 from test_gpu_mlp import _gradient_parity, _setup  # noqa: F401  (_setup is the module's fixture)
 
@@ -37,7 +39,15 @@ def test_both_sides_of_the_small_product_rule(workers):
     _gradient_parity([512, 512, 10], 128, sim.GEM_MLP_FP32, 1e-5, 1e-5, 3, workers)
 
 
-# TF32 products that the tensor cores do not take: fewer than 32 rows or a K below 32
-@pytest.mark.parametrize("dims,b", [([784, 64, 10], 8), ([100, 31, 10], 31), ([96, 40, 16], 64)])
+# TF32 products that the tensor cores do not take: fewer than 32 rows or a K below 32, and those
+# of small networks
+@pytest.mark.parametrize("dims,b", [([784, 64, 10], 8), ([100, 31, 10], 31), ([96, 40, 16], 64),
+                                    ([300, 130, 65, 10], 130), ([516, 384, 10], 128)])
 def test_tf32_small_products_match_oracle(dims, b):
     _gradient_parity(dims, b, sim.GEM_MLP_TF32, 1e-4, 1e-2, 3, [1, 0])
+
+
+def test_tf32_tiles_96_wide():
+    """13 workers of 1,000 columns: 143 tiles 96-wide, the last one of a row 40 columns, on K with
+    a remainder (the bars of the wide layers in test_gpu_mlp)."""
+    _gradient_parity([100, 1000, 516, 10], 128, sim.GEM_MLP_TF32, 3e-4, 1e-2, 13, list(range(13)))
