@@ -1116,11 +1116,13 @@ int gem_cnn_grad(gem_cnn_t* N, const int32_t* workers, int L, const int32_t* bat
   cudaSetDevice(h->device);
   int rc = upload_rows(N, batch_rows, (long long)L * N->batch);
   const long long db = (long long)N->batch * N->sh.c2;
+  const long long spacing = gem::mlp::row_spacing(grads, L, h->P);
   for (int c0 = 0; c0 < L && rc == GEM_OK; c0 += N->slots) {
     const int G = (L - c0) < N->slots ? (L - c0) : N->slots;
     rc = cnn_chunk(N, workers + c0, G, N->rows_dev + (long long)c0 * N->batch, drop + c0 * db,
-                   N->grads, (long long)h->stride, losses ? losses + c0 : nullptr);
-    for (int g = 0; g < G && rc == GEM_OK; ++g)
+                   spacing ? grads[c0] : N->grads, spacing ? spacing : (long long)h->stride,
+                   losses ? losses + c0 : nullptr);
+    for (int g = 0; !spacing && g < G && rc == GEM_OK; ++g)
       rc = cuda_rc(cudaMemcpyAsync(grads[c0 + g], N->grads + (long long)g * h->stride,
                                    h->P * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
   }

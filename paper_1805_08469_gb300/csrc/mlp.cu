@@ -2022,6 +2022,22 @@ void mlp_free(gem_mlp* M) {
 }  // namespace mlp
 }  // namespace gem
 
+namespace gem {
+namespace mlp {
+
+long long row_spacing(float* const* rows, int n, size_t P) {
+  if (n < 2) return n == 1 ? (long long)((P + 3) / 4 * 4) : 0;
+  const uintptr_t first = reinterpret_cast<uintptr_t>(rows[0]);
+  const uintptr_t second = reinterpret_cast<uintptr_t>(rows[1]);
+  if (second <= first || (second - first) % 16 != 0 || (second - first) / sizeof(float) < P) return 0;
+  for (int i = 2; i < n; ++i)
+    if (reinterpret_cast<uintptr_t>(rows[i]) != first + uintptr_t(i) * (second - first)) return 0;
+  return (long long)((second - first) / sizeof(float));
+}
+
+}  // namespace mlp
+}  // namespace gem
+
 namespace {
 
 // Check minibatch rows on the host and copy them to the device (stream-ordered).
@@ -2108,11 +2124,12 @@ int gem_mlp_grad(gem_mlp_t* M, const int32_t* workers, int L, const int32_t* bat
   cudaGetDevice(&dev_prev);
   cudaSetDevice(h->device);
   int rc = upload_rows(M, batch_rows, (long long)L * M->batch);
+  const long long spacing = gem::mlp::row_spacing(grads, L, h->P);
   for (int c0 = 0; c0 < L && rc == GEM_OK; c0 += M->slots) {
     const int G = (L - c0) < M->slots ? (L - c0) : M->slots;
-    rc = mlp_chunk(M, workers + c0, G, M->rows_dev + (long long)c0 * M->batch, M->grads,
-                   (long long)h->stride, losses ? losses + c0 : nullptr);
-    for (int g = 0; g < G && rc == GEM_OK; ++g)
+    rc = mlp_chunk(M, workers + c0, G, M->rows_dev + (long long)c0 * M->batch, spacing ? grads[c0] : M->grads,
+                   spacing ? spacing : (long long)h->stride, losses ? losses + c0 : nullptr);
+    for (int g = 0; !spacing && g < G && rc == GEM_OK; ++g)
       rc = cuda_rc(cudaMemcpyAsync(grads[c0 + g], M->grads + (long long)g * h->stride,
                                    h->P * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
   }

@@ -89,6 +89,11 @@ void mlp_free(gem_mlp* M);
 int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_rows,
               float* grads, long long grad_stride, float* losses);
 
+// The spacing in floats of n caller rows of P floats that lie one after the other at equal
+// distances (rows of one buffer, say), or 0: gradients then go to the caller's rows directly
+// instead of through the handle's and a copy each.
+long long row_spacing(float* const* rows, int n, size_t P);
+
 inline float* mlp_input(gem_mlp* M, int g) { return M->scratch + g * M->slot_stride + M->off_x; }
 inline float* mlp_input_grad(gem_mlp* M, int g) {
   return M->scratch + g * M->slot_stride + M->off_delta[0];

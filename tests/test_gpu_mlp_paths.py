@@ -47,6 +47,38 @@ def test_tf32_small_products_match_oracle(dims, b):
     _gradient_parity(dims, b, sim.GEM_MLP_TF32, 1e-4, 1e-2, 3, [1, 0])
 
 
+@pytest.mark.parametrize("layout", ["rows", "spaced", "reversed", "scattered", "one"])
+def test_gradients_are_the_same_wherever_the_caller_wants_them(layout):
+    """Equally spaced rows are written in place, others through a copy: the same values, and
+    nothing outside the P floats of a row."""
+    dims, b, seed = [40, 37, 10], 20, 5
+    P = synth.mlp_param_count(dims)
+    workers = [2, 0, 1] if layout != "one" else [1]
+    ld = (P + 3) // 4 * 4 + (64 if layout == "spaced" else 0)
+    X = torch.empty((300, dims[0]), device="cuda")
+    y = torch.empty(300, dtype=torch.int32, device="cuda")
+    synth_gpu.data(seed, X, y, 10)
+    rows = np.random.default_rng(1).integers(0, 300, (len(workers), b)).astype(np.int32)
+    buf = torch.full((8, ld), -7.0, device="cuda")
+    at = {"rows": [0, 1, 2], "spaced": [1, 3, 5], "reversed": [2, 1, 0], "scattered": [0, 5, 3], "one": [4]}[layout]
+    with gem.Gem(P, 3, 0.01, 0.9, 1e-8) as G:
+        G.set_theta(synth_gpu.xavier(seed, dims, torch.empty(P, device="cuda")))
+        M = sim.gem_mlp_create(G.h, dims, b)
+        sim.gem_mlp_set_data(M, X, y)
+        apart = [torch.empty(P, device="cuda") for _ in range(2 * len(workers))][::2]
+        sim.gem_mlp_grad(M, workers, rows, [buf[i, :P] for i in at])
+        for k, w in enumerate(workers):        # one worker at a time
+            sim.gem_mlp_grad(M, [w], rows[k:k + 1], [apart[k]])
+        sim.gem_mlp_status(M)
+        sim.gem_mlp_destroy(M)
+    for k, i in enumerate(at):
+        assert torch.allclose(buf[i, :P], apart[k], rtol=0, atol=1e-6 * float(apart[k].abs().max()))
+    mask = torch.ones_like(buf, dtype=torch.bool)
+    for i in at:
+        mask[i, :P] = False
+    assert bool((buf[mask] == -7.0).all())
+
+
 def test_tf32_tiles_96_wide():
     """13 workers of 1,000 columns: 143 tiles 96-wide, the last one of a row 40 columns, on K with
     a remainder (the bars of the wide layers in test_gpu_mlp)."""
