@@ -117,6 +117,12 @@ __global__ void count_init_kernel(const __grid_constant__ CountInitArgs a) {
   if (i <= a.nseg) a.seg_dev[i] = a.seg[i];
 }
 
+// HBM and the shared-memory atomics bound it: whole steps of 2,048 elements have no bounds
+// checks, and one comparison per element while the targets share their prefix.  64 rows of 5M
+// factors in six segments, a third of them settled before (us): first pass 266 with a match of
+// the warp's digits before the atomics, 87 without it, 58 without the checks; later passes 88,
+// 109 and 60.  Blocks of 131,072 elements instead of 16,384 took 148 and 195: too few of them
+// have a segment that is not settled.
 template <bool FIRST>
 __global__ void __launch_bounds__(kThreads) select_hist_kernel(const __grid_constant__ SelectArgs a) {
   gem::pdl_entry();
@@ -140,26 +146,29 @@ __global__ void __launch_bounds__(kThreads) select_hist_kernel(const __grid_cons
   const long long end = beg + kChunk < a.seg[s + 1] ? beg + kChunk : a.seg[s + 1];
   const float* x = a.pi[k];
   unsigned zeros = 0u;   // first pass: this thread's elements equal to +0
-  for (long long base = beg; base < end; base += kThreads * kUnroll) {
+  // one prefix to match unless the targets have parted: then the second goes to its own bins
+  const unsigned pa = need0 ? p0 : p1, ma = need0 ? m0 : m1;
+  unsigned* ha = need0 ? h : h + kBins;
+  const bool both = need0 && need1;
+  auto count = [&](unsigned key) {
+    const unsigned d = (key >> shift) & dmask;
+    if (FIRST) {
+      if (key == kZeroKey) ++zeros;
+      else atomicAdd(h + d, 1u);
+    } else {
+      if ((key & ma) == pa) atomicAdd(ha + d, 1u);
+      if (both && (key & m1) == p1) atomicAdd(h + kBins + d, 1u);
+    }
+  };
+  long long base = beg;
+  for (; base + kThreads * kUnroll <= end; base += kThreads * kUnroll) {
     unsigned key[kUnroll];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const long long i = base + u * kThreads + threadIdx.x;
-      key[u] = i < end ? order_key(x[i]) : 0u;
-    }
+    for (int u = 0; u < kUnroll; ++u) key[u] = order_key(x[base + u * kThreads + threadIdx.x]);
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      if (base + u * kThreads + threadIdx.x >= end) continue;
-      const unsigned d = (key[u] >> shift) & dmask;
-      if (FIRST) {
-        if (key[u] == kZeroKey) ++zeros;
-        else atomicAdd(h + d, 1u);
-      } else {
-        if (need0 && (key[u] & m0) == p0) atomicAdd(h + d, 1u);
-        if (need1 && (key[u] & m1) == p1) atomicAdd(h + kBins + d, 1u);
-      }
-    }
+    for (int u = 0; u < kUnroll; ++u) count(key[u]);
   }
+  for (long long i = base + threadIdx.x; i < end; i += kThreads) count(order_key(x[i]));
   if (FIRST) {
     zeros = __reduce_add_sync(0xffffffffu, zeros);
     if ((threadIdx.x & 31) == 0 && zeros) atomicAdd(h + kBins, zeros);
@@ -262,8 +271,9 @@ constexpr int kSmallUnroll = 16;            // independent loads per thread and 
 // memory.  The factors are read once (L2 serves them: the commit has just written them), 16
 // loads per thread in flight; each pass counts digits with shared-memory atomics, scans the
 // bins with the whole block, two per thread, and extends the targets' prefixes.
-// What bounds it is the latency of that chain.  Measured, the MNIST network with n = 30 and its ten
-// tensors (up to 40,960 factors): see commit_pi_median_ordered.
+// What bounds it is the latency of that chain.  Measured, the MNIST network with n = 30, whose ten
+// tensors have up to 40,960 factors: 24 us per segment instead of 75 for eight launches
+// (cold), 32 commits 1,166 -> 949 us.
 __global__ void __launch_bounds__(kSmallThreads) select_small_kernel(const __grid_constant__ SelectArgs a) {
   gem::pdl_entry();
   extern __shared__ unsigned small_smem[];
