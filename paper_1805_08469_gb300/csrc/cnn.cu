@@ -15,9 +15,12 @@
 //   conv2_wpart_kernel,    per-sample partial sums of the convolution weight and bias
 //   conv1_wpart_kernel     gradients
 //   conv_finish_kernel     sums of the partials over the minibatch, in sample order
+// Networks of the paper's map sizes (28 x 28 inputs) whose staging fits run the *28 forms of the
+// convolution kernels, which share a worker's weights among several samples of a block and
+// sum in the same order; other shapes run the general ones.
 // Every value is summed in a fixed order, so the gradients do not depend on timing.  The
-// per-sample kernels stage a sample's maps and the worker's weights in shared memory; a
-// shape whose staging exceeds 160 KB is refused.
+// general kernels stage a sample's maps and the worker's weights in shared memory; a
+// shape whose staging there exceeds 160 KB is refused.
 #include <cstdint>
 #include <cstring>
 #include <new>

@@ -16,9 +16,13 @@
 //   biases    db_l = column sums of D_{l+1} (fixed order, no atomics)
 // Every sum runs in a fixed order, so the gradients are deterministic.
 //
-// Precision.  Every product runs in one grouped SIMT GEMM kernel that reads either operand
-// layout; with GEM_MLP_TF32 it rounds each operand to TF32 as it loads it (products of TF32
-// values are exact in fp32; the sums stay fp32).
+// Precision.  With GEM_MLP_FP32 every product runs on the CUDA cores: gemm_grouped_kernel where
+// the FMAs bound it, gemm_simt_kernel (small products, the splits of K in one cluster) and
+// weight_grad_kernel (a small network's weight and bias gradients) where latency does; the
+// order of the sums is that of the product, not of the kernel.  With GEM_MLP_TF32 each operand is
+// rounded to TF32 (products of TF32 values are exact in fp32; the sums stay fp32): on the
+// tensor cores (tc_gemm.cu, and mma.sync here), small networks and small products on the CUDA
+// cores (launch_gemm).
 #include <cooperative_groups.h>
 #include <cuda.h>
 
