@@ -90,6 +90,7 @@ struct BatchArgsT {
   const long long* pi_seg;                 // device array [pi_nseg + 1], non-decreasing
   int pi_nseg;
   int lane_rows;                           // dynamic shared memory: rows of a 16-byte lane per thread
+  int grads_through_l1;                    // 1: the copies of the gradients are cached in L1
 };
 using BatchArgs = BatchArgsT<kMaxBatchPerLaunch>;
 constexpr int kSmallBatch = 32;

@@ -100,3 +100,30 @@ def test_batches_equal_single_commits(P, rule):
         assert torch.equal(A.theta(), B.theta())
         for w in range(n):
             assert torch.equal(A.snapshot(w), B.snapshot(w)) and torch.equal(A.moment(w), B.moment(w))
+
+
+# Gradient rows on 128-byte lines and between them (every row of a launch, or one), and each
+# remainder of a ragged row.
+@pytest.mark.parametrize("P", [3, 510, 4097, 200_003])
+@pytest.mark.parametrize("offsets", [(0,), (4,), (28,), (0, 0, 12)])
+@pytest.mark.parametrize("rule", [0, 1, 5])
+def test_gradient_rows_at_every_alignment(P, offsets, rule):
+    rng = np.random.default_rng(P)
+    ld = (P + 31) // 32 * 32 + 32
+    pool = torch.zeros((6, ld), device="cuda")
+    pool.copy_(torch.from_numpy((0.1 * rng.standard_normal((6, ld))).astype(np.float32)))
+    assert pool.data_ptr() % 128 == 0
+    rows = [pool[i, o:o + P] for i, o in zip(range(6), offsets * 6)]
+    order = [0, 1, 2, 0, 0, 1]
+    with gem.Gem(P, 3, 0.01, 0.9, 1e-8) as A, gem.Gem(P, 3, 0.01, 0.9, 1e-8) as B:
+        for G in (A, B):
+            G.set_theta(torch.from_numpy(rng.standard_normal(P).astype(np.float32)).cuda() if G is A else A.theta().clone())
+            G.set_mode(rule, 1.5)
+        A.commit_batch(order, rows)
+        for w, g in zip(order, rows):
+            B.commit(w, g.clone())
+        A.sync()
+        B.sync()
+        assert torch.equal(A.theta(), B.theta())
+        for w in range(3):
+            assert torch.equal(A.snapshot(w), B.snapshot(w)) and torch.equal(A.moment(w), B.moment(w))
