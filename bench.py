@@ -52,8 +52,8 @@ FALLBACK_HBM_GBS = 6800.0
 # on the device), scaled by P: the traffic per coordinate does not depend on P (captures at
 # P = 2,500,000 and 5,000,000 agree within 1%).  Valid only for the kernel source it was
 # taken on (NCU_TRAFFIC_SOURCE_SHA, a hash of the kernel's sources); null once that changes.
-NCU_TRAFFIC_BYTES_PER_LAUNCH = 5 * (7_422_780_416 + 7_097_482_752) // 2   # mean of two launches at P = 5M
-NCU_TRAFFIC_SOURCE_SHA = "ddbcc0bf230bd62b"
+NCU_TRAFFIC_BYTES_PER_LAUNCH = 5 * (7_422_885_632 + 7_097_584_640) // 2   # mean of two launches at P = 5M
+NCU_TRAFFIC_SOURCE_SHA = "865f1023c6c530fb"
 NCU_TRAFFIC_HOW = "two launches captured at P=5,000,000 (n=100, K=100), scaled by P to 25,000,000"
 
 
