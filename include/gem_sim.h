@@ -63,8 +63,7 @@ enum gem_mlp_precision {
                        tcgen05 tensor cores where both operands are K-major (forward
                        products; weight gradients through transposed minibatch panels),
                        on warp-level mma.sync for the input gradients, and on the CUDA
-                       cores, with the same rounding, below 32 rows or a K of 32 and in
-                       small networks (no product above 40 million multiply-adds) */
+                       cores, with the same rounding, below 32 rows or a K of 32 */
 };
 
 /* Bind an MLP to a GEM handle (its P must equal the MLP's parameter count).  batch is the

@@ -21,7 +21,7 @@
 // weight_grad_kernel (a small network's weight and bias gradients) where latency does; the
 // order of the sums is that of the product, not of the kernel.  With GEM_MLP_TF32 each operand is
 // rounded to TF32 (products of TF32 values are exact in fp32; the sums stay fp32): on the
-// tensor cores (tc_gemm.cu, and mma.sync here), small networks and small products on the CUDA
+// tensor cores (tc_gemm.cu, and mma.sync here), products of few rows or a short K on the CUDA
 // cores (launch_gemm).
 #include <cooperative_groups.h>
 #include <cuda.h>
@@ -94,7 +94,6 @@ struct GemmArgs {
   float* ws;            // null: no split
   long long ws_floats;  // capacity of ws
   int can_split;        // CUDA-core path: K may be cut
-  int cuda_cores;       // TF32: take the CUDA-core path
   // tensor-core path: floats addressable from each operand's base (0: unknown, which keeps
   // the product off that path) and the error word its kernels report to
   long long a_extent, b_extent, c_extent, bias_extent, mask_extent;
@@ -1354,7 +1353,6 @@ struct WeightGradArgs {
   long long grad_stride;
 };
 
-template <bool TF32>
 __global__ void __launch_bounds__(kSimtThreads, 4)
 weight_grad_kernel(const __grid_constant__ WeightGradArgs w, const __grid_constant__ BiasGradArgs bias) {
   gem::pdl_entry();
@@ -1379,7 +1377,7 @@ weight_grad_kernel(const __grid_constant__ WeightGradArgs w, const __grid_consta
   const SimtOperand B = l == 0 && w.X ? SimtOperand{w.X, N, w.batch_rows + (long long)g * w.b, w.b}
                                       : SimtOperand{slot + w.off_act[l], N, nullptr, 0};
   float acc[Tile::TM][Tile::TN];
-  simt_tile<BM, false, false, TF32>(A, B, M, N, m0, n0, 0, w.b, simt_smem, row_idx, acc);
+  simt_tile<BM, false, false, false>(A, B, M, N, m0, n0, 0, w.b, simt_smem, row_idx, acc);
   const int tx = threadIdx.x % Tile::TX, ty = threadIdx.x / Tile::TX;
   float* C = w.grads + g * w.grad_stride + w.w_off[l];
   const int n = n0 + 4 * tx;
@@ -1539,10 +1537,9 @@ cudaError_t launch_gemm(const GemmArgs& a_in, int groups, bool tf32, cudaStream_
   a.ksplit = 1;
   a.kchunk = a.K;
   // Products with fewer than 32 rows or a K below 32 (the last layer's weight and input
-  // gradients) would leave a 128-row tensor-core tile mostly empty or its pipeline idle, and
-  // those of a small network (a.cuda_cores) are over before a tensor-core kernel has set itself
-  // up: they run on the CUDA cores, with the same TF32 operand rounding.
-  const bool tc = tf32 && a.M >= 32 && a.K >= 32 && !a.cuda_cores;
+  // gradients) would leave a 128-row tensor-core tile mostly empty or its pipeline idle:
+  // they run on the CUDA cores, with the same TF32 operand rounding.
+  const bool tc = tf32 && a.M >= 32 && a.K >= 32;
   if (!tc)
     return tf32 ? launch_cuda_cores<AK, BK_, EPI, true>(a, groups, st)
                 : launch_cuda_cores<AK, BK_, EPI, false>(a, groups, st);
@@ -1630,16 +1627,10 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   auto act = [&](int l) -> float* { return l == 0 ? scr + M->off_x : scr + M->off_act[l]; };
 
   int rc = GEM_OK;
-  // Small networks, whose every weight gradient (and so every product) is small: CUDA cores also
-  // with TF32 operands, and the weight and bias gradients in one launch (below).  TF32, whole runs
-  // with the tensor cores and with this: 130-118-10, b = 40, 20 commits 245 and 189 us; 62-27-16-
-  // 30-10, b = 96 498 and 332; 784-54-948-10, b = 46 1,722 and 1,521.
-  bool small = true;
-  for (int l = 0; l < L; ++l) small = small && small_product(M->dims[l + 1], M->dims[l], b, G);
   // the minibatch rows: read in place by the small products of the first layer (its forward
-  // product and its weight gradient have the same size), gathered for the others (rounded with
-  // TF32 operands)
-  const bool in_place = !M->external_input && (small || (!tf32 && small_product(b, M->dims[1], M->dims[0], G)));
+  // product and its weight gradient have the same size), gathered for the others (rounded for
+  // the tensor cores)
+  const bool in_place = !M->external_input && !tf32 && small_product(b, M->dims[1], M->dims[0], G);
   if (!M->external_input && !in_place) {
     gem::launch_pdl(gather_rows_kernel, dim3(b, G), 256, 0, st, M->X, M->dims[0], batch_rows, b,
                                                    scr + M->off_x, S, tf32 ? 1 : 0);
@@ -1653,7 +1644,6 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   a.ws = M->ws;
   a.ws_floats = M->ws_floats;
   a.can_split = b <= 128 && M->scratch_end != nullptr;
-  a.cuda_cores = small ? 1 : 0;
   a.status = M->tc_status;
   const long long wstride = (long long)h->stride;
   // floats addressable from p when it lies in the scratch or in the snapshots (0 otherwise)
@@ -1680,14 +1670,14 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   // rounding again): the gathered rows (rounded by the gather) and activations stored
   // rounded by a tensor-core forward product.
   bool act_rnd[kMaxLayers + 1] = {};
-  act_rnd[0] = tf32 && !M->external_input && !in_place;
+  act_rnd[0] = tf32 && !M->external_input;
   // Weight gradients dW_l = D_{l+1}^T A_l that run on the tensor cores read the minibatch
   // panels K-major (K = the batch): TF32-rounded transposes A_l^T and D_{l+1}^T.  A hidden
   // activation's transpose comes from the epilogue of the tensor-core product that makes it;
   // X^T and the deltas' transposes from transpose_round_kernel on the side stream, next to
   // the main stream's chain.
   auto t_dw = [&](int l) {
-    return M->has_t && !small && l + 1 < L && M->dims[l + 1] >= 32 && b >= 32 && b % 4 == 0;
+    return M->has_t && l + 1 < L && M->dims[l + 1] >= 32 && b >= 32 && b % 4 == 0;
   };
   TransposeArgs ta;
   std::memset(&ta, 0, sizeof(ta));
@@ -1792,7 +1782,9 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   // Small networks: the weight and bias gradients in one launch, once the deltas are known; on
   // the main stream, or on the side stream next to the input gradient and what the caller
   // does with it.
-  const bool aside = small && two_streams && M->input_grad;
+  bool merged = !tf32;
+  for (int l = 0; l < L; ++l) merged = merged && small_product(M->dims[l + 1], M->dims[l], b, G);
+  const bool aside = merged && two_streams && M->input_grad;
   auto weight_grads = [&]() -> int {
     WeightGradArgs wa;
     std::memset(&wa, 0, sizeof(wa));
@@ -1818,9 +1810,8 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
       if (r == GEM_OK) r = cuda_rc(cudaStreamWaitEvent(wst, M->ev_delta[1], 0));
       if (r) return r;
     }
-    gem::launch_pdl(tf32 ? weight_grad_kernel<true> : weight_grad_kernel<false>,
-                    dim3(unsigned(wa.first[L] + (ba.first[L] + 31) / 32), unsigned(G)), kSimtThreads, size_t(bytes),
-                    aside ? wst : st, wa, ba);
+    gem::launch_pdl(weight_grad_kernel, dim3(unsigned(wa.first[L] + (ba.first[L] + 31) / 32), unsigned(G)),
+                    kSimtThreads, size_t(bytes), aside ? wst : st, wa, ba);
     M->launches++;
     return cuda_rc(cudaGetLastError());
   };
@@ -1830,7 +1821,7 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   // to the input-gradient chain; they use no split-K workspace, which belongs to the main stream.
   for (int l = L - 1; l >= 0; --l) {
     const int din = M->dims[l], dout = M->dims[l + 1];
-    if (small) {
+    if (merged) {
       if (l == 0 && (rc = weight_grads())) return rc;
     } else {
       if (two_streams) {
@@ -1907,13 +1898,13 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
     if ((rc = cuda_rc(launch_gemm<true, false, kMask>(a, G, tf32, st)))) return rc;
     M->launches++;
   }
-  if (!small) {
+  if (!merged) {
     gem::launch_pdl(bias_grad_kernel, dim3((ba.first[L] + 31) / 32, G), 256, 0, st, ba, scr, S, grads,
                     grad_stride);
     if ((rc = cuda_rc(cudaGetLastError()))) return rc;
     M->launches++;
   }
-  if (two_streams && (!small || aside)) {   // the gradients are complete once the side stream is
+  if (two_streams && (!merged || aside)) {   // the gradients are complete once the side stream is
     if ((rc = cuda_rc(cudaEventRecord(M->ev_side, wst)))) return rc;
     if ((rc = cuda_rc(cudaStreamWaitEvent(st, M->ev_side, 0)))) return rc;
   }

@@ -39,10 +39,8 @@ def test_both_sides_of_the_small_product_rule(workers):
     _gradient_parity([512, 512, 10], 128, sim.GEM_MLP_FP32, 1e-5, 1e-5, 3, workers)
 
 
-# TF32 products that the tensor cores do not take: fewer than 32 rows or a K below 32, and those
-# of small networks
-@pytest.mark.parametrize("dims,b", [([784, 64, 10], 8), ([100, 31, 10], 31), ([96, 40, 16], 64),
-                                    ([300, 130, 65, 10], 130), ([516, 384, 10], 128)])
+# TF32 products that the tensor cores do not take: fewer than 32 rows or a K below 32
+@pytest.mark.parametrize("dims,b", [([784, 64, 10], 8), ([100, 31, 10], 31), ([96, 40, 16], 64)])
 def test_tf32_small_products_match_oracle(dims, b):
     _gradient_parity(dims, b, sim.GEM_MLP_TF32, 1e-4, 1e-2, 3, [1, 0])
 
