@@ -70,8 +70,9 @@ struct Operand {
   long long group_stride;  // elements between the operands of consecutive groups
   long long ld;            // leading dimension of its row-major storage
   int by_worker;           // group g uses index workers[g] (GEM state) instead of g (scratch)
-  // CUDA-core path only: storage row r of group g is row rows[g * rows_per_group + r] of base
-  // (minibatch rows read in place from the data set); null: row r of group g's operand
+  // gemm_simt_kernel only (the launchers of the other kernels refuse such an operand): storage
+  // row r of group g is row rows[g * rows_per_group + r] of base (minibatch rows read in place
+  // from the data set); null: row r of group g's operand
   const int32_t* rows;
   int rows_per_group;
 };
@@ -1139,6 +1140,10 @@ gemm_small_n_kernel(const __grid_constant__ GemmArgs p, int rows_per_block,
 template <bool TF32>
 bool launch_small_n(const GemmArgs& a, int groups, cudaStream_t st, cudaError_t* err,
                     const XentArgs* xent) {
+  if (a.A.rows || a.B.rows) {   // the kernel does not read through row indices
+    *err = cudaErrorInvalidValue;
+    return true;
+  }
   const size_t bytes = sizeof(float) * size_t(a.N) * size_t(a.K);
   constexpr size_t kMaxBytes = 200 * 1024;
   if (bytes > kMaxBytes) return false;
@@ -1490,6 +1495,7 @@ cudaError_t launch_cuda_cores(GemmArgs a, int groups, cudaStream_t st) {
   a.ksplit = simt_split(a.M, a.N, a.K, groups, a.can_split != 0);
   a.kchunk = a.ksplit > 1 ? ((a.K + a.ksplit - 1) / a.ksplit + BK - 1) / BK * BK : a.K;
   if (small_product(a.M, a.N, a.K, groups)) return launch_simt<AK, BK_, EPI, TF32>(a, groups, st);
+  if (a.A.rows || a.B.rows) return cudaErrorInvalidValue;   // gemm_grouped_kernel reads no row indices
   const long long big = (long long)((a.N + BN - 1) / BN) * ((a.M + 127) / 128) * groups;
   if (big >= GEM_SIMT_BIG_TILE_BLOCKS * kSmCountHint) {
     launch_tile<128, AK, BK_, EPI, TF32>(a, groups, st);
@@ -1543,6 +1549,7 @@ cudaError_t launch_gemm(const GemmArgs& a_in, int groups, bool tf32, cudaStream_
   if (!tc)
     return tf32 ? launch_cuda_cores<AK, BK_, EPI, true>(a, groups, st)
                 : launch_cuda_cores<AK, BK_, EPI, false>(a, groups, st);
+  if (a.A.rows || a.B.rows) return cudaErrorInvalidValue;   // nor do the tensor-core kernels
   if (a.a_extent > 0 && a.b_extent > 0 && a.c_extent > 0) {
     // the 5th-generation tensor cores (tcgen05, accumulator in tensor memory), for products
     // whose layout, epilogue and alignment its kernel takes; the others stay on mma.sync
@@ -1629,8 +1636,9 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
   int rc = GEM_OK;
   // the minibatch rows: read in place by the small products of the first layer (its forward
   // product and its weight gradient have the same size), gathered for the others (rounded for
-  // the tensor cores)
-  const bool in_place = !M->external_input && !tf32 && small_product(b, M->dims[1], M->dims[0], G);
+  // the tensor cores).  The forward product of a network with one layer is the logits kernel,
+  // which reads gathered rows.
+  const bool in_place = !M->external_input && !tf32 && L > 1 && small_product(b, M->dims[1], M->dims[0], G);
   if (!M->external_input && !in_place) {
     gem::launch_pdl(gather_rows_kernel, dim3(b, G), 256, 0, st, M->X, M->dims[0], batch_rows, b,
                                                    scr + M->off_x, S, tf32 ? 1 : 0);

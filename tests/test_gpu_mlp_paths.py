@@ -8,9 +8,10 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_1805_08469_gb300 import gem, sim, synth, synth_gpu
 
-from test_gpu_mlp import _gradient_parity, _setup  # noqa: F401  (_setup is the module's fixture)
+from test_gpu_mlp import _gradient_parity, _setup, rel_l2, theta0_with_biases  # noqa: F401  (_setup is the module's fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -81,3 +82,54 @@ def test_tf32_tiles_96_wide():
     """13 workers of 1,000 columns: 143 tiles 96-wide, the last one of a row 40 columns, on K with
     a remainder (the bars of the wide layers in test_gpu_mlp)."""
     _gradient_parity([100, 1000, 516, 10], 128, sim.GEM_MLP_TF32, 3e-4, 1e-2, 13, list(range(13)))
+
+
+# A network without a hidden layer: its first product is also the logits.  The rows of a minibatch
+# are in random order with repeats, and with 3 rows the data set is shorter than the minibatch.
+@pytest.mark.parametrize("dims", [[784, 10], [37, 3], [40, 37, 10]])
+@pytest.mark.parametrize("precision", [sim.GEM_MLP_FP32, sim.GEM_MLP_TF32])
+@pytest.mark.parametrize("b,rows", [(1, 500), (33, 500), (128, 500), (33, 3)])
+def test_minibatch_rows_of_every_entry_point(dims, precision, b, rows):
+    """gem_mlp_grad, gem_mlp_grad_static and gem_mlp_run read the rows that they are given.  The
+    bars are those of test_gpu_mlp: 1e-5 for fp32 products and, with TF32 operands, 1e-2
+    where the delta is rounded, 1e-4 for the loss; theta 1e-4 and 2e-3."""
+    seed, n, T = 11, 3, 7
+    tf32 = precision == sim.GEM_MLP_TF32
+    bar, deep = (1e-4, 1e-2) if tf32 else (1e-5, 1e-5)
+    P = synth.mlp_param_count(dims)
+    rng = np.random.default_rng(rows + b)
+    X = rng.standard_normal((rows, dims[0])).astype(np.float32)
+    y = rng.integers(0, dims[-1], rows).astype(np.int32)
+    order = rng.integers(0, n, T).astype(np.int32)
+    batches = rng.integers(0, rows, (T, b)).astype(np.int32)
+    theta0 = theta0_with_biases(seed, dims)
+    Xd, yd, td = torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda(), torch.from_numpy(theta0).cuda()
+    got = [torch.empty((P + 3) // 4 * 4, device="cuda")[:P] for _ in range(2 * n)]
+    losses = torch.empty(2 * n, device="cuda")
+    run_losses = torch.empty(T, device="cuda")
+    with gem.Gem(P, n, 0.01, 0.9, 1e-8) as G:
+        G.set_theta(td)
+        M = sim.gem_mlp_create(G.h, dims, b, precision)
+        try:
+            sim.gem_mlp_set_data(M, Xd, yd)
+            sim.gem_mlp_grad(M, list(range(n)), batches[:n], got[:n], losses)
+            G.sync()
+            for k in range(n):
+                sim.gem_mlp_grad_static(dims, b, precision, td, Xd, yd, batches[k], got[n + k], losses[n + k:])
+            torch.cuda.synchronize()
+            sim.gem_mlp_run(M, order, batches, run_losses)
+            G.sync()
+            theta = G.theta().cpu().numpy()
+            sim.gem_mlp_status(M)
+        finally:
+            sim.gem_mlp_destroy(M)
+    for k in range(2 * n):
+        r = batches[k % n]
+        loss, g = oracle.mlp_loss_grad(dims, theta0.astype(np.float64), X[r], y[r], tf32=tf32)
+        assert rel_l2(got[k].cpu().numpy(), g) < deep, k
+        assert abs(float(losses[k]) - loss) <= bar * abs(loss) + 1e-6, k
+    th, m, s = theta0.copy(), np.zeros((n, P), np.float32), np.tile(theta0, (n, 1))
+    _r, ref = oracle.mlp_sim_run(dims, th, m, s, order, X, y, batches, eta=0.01, mu=0.9, eps=1e-8, tf32=tf32,
+                                 want_losses=True)
+    assert rel_l2(theta, th) < (2e-3 if tf32 else 1e-4)
+    np.testing.assert_allclose(run_losses.cpu().numpy(), ref, rtol=2e-3 if tf32 else 1e-4)
