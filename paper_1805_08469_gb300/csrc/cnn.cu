@@ -84,6 +84,7 @@ int cuda_rc(cudaError_t e) { return e == cudaSuccess ? GEM_OK : GEM_ECUDA; }
 
 struct ConvArgs {
   int H, c1, c2, H1, P1, H2, P2, F, b, G;
+  int pool2_per, back_per;     // samples per block of conv2_pool28_kernel and conv2_back28_kernel
   const float* X;              // [rows][H * H]
   const int32_t* rows;         // [G][b] minibatch rows
   const float* snap;           // GEM snapshots s, [n][snap_stride]
@@ -473,8 +474,11 @@ __global__ void __launch_bounds__(kW1Threads) conv1_wpart_kernel(const __grid_co
 // 16.3; the run of n = 100 1,081 -> 847 us.
 constexpr int kH = 28, kH1 = 24, kP1 = 12, kH2 = 8, kP2 = 4;   // map sides
 constexpr int kWPitch = 28;                                    // floats per kernel of 25 weights
-constexpr int kPer28 = 2;                                      // samples per block of conv2_pool28_kernel
-constexpr int kBackPer28 = 3;                                  // the same of conv2_back28_kernel
+// samples per block of conv2_pool28_kernel and conv2_back28_kernel (ConvArgs::pool2_per and
+// back_per), or one while that gives no SM a second block: sharing the weights then only makes
+// blocks longer.  Gradients of 16 and 64 channels, b = 64, 2 workers 190 us with 2 and 3, 138 with
+// one; 10 and 20 channels 84 and 79
+constexpr int kPer28 = 2, kBackPer28 = 3;
 // floats between the channels of a map in shared memory where the lanes of a quarter-warp read
 // 16 bytes each of different channels: 576 + 4, and 144 + 12, for which (channel, row) in turn
 // step by 12 floats mod 32; the plain strides gave 7- and 2-way bank conflicts
@@ -560,19 +564,19 @@ __global__ void __launch_bounds__(kPool1Threads28) conv1_pool28_kernel(const __g
   }
 }
 
-// conv2 + bias, dropout scale, pool, ReLU: a block per kPer28 samples of a worker, 16 threads per
+// conv2 + bias, dropout scale, pool, ReLU: a block per pool2_per samples of a worker, 16 threads per
 // pair of output channels and sample, a thread per window, which keeps its patch for both.
 constexpr int kPool2Threads28 = 320;
 __global__ void __launch_bounds__(kPool2Threads28) conv2_pool28_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ __align__(16) float sm[];
-  const int per_g = (a.b + kPer28 - 1) / kPer28;
-  const int g = blockIdx.x / per_g, i0 = (blockIdx.x - g * per_g) * kPer28;
-  const int ns = min(kPer28, a.b - i0);
+  const int per = a.pool2_per, per_g = (a.b + per - 1) / per;
+  const int g = blockIdx.x / per_g, i0 = (blockIdx.x - g * per_g) * per;
+  const int ns = min(per, a.b - i0);
   const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
   const int n_a1 = a.c1 * kP1 * kP1;
   float* ws = sm;                                   // [c2][c1][28]
-  float* a1s = ws + a.c2 * a.c1 * kWPitch;          // [kPer28][c1][12][12]
+  float* a1s = ws + a.c2 * a.c1 * kWPitch;          // [pool2_per][c1][12][12]
   stage(a1s, a.scr + g * a.S + a.o_a1 + (long long)i0 * n_a1, ns * n_a1);
   stage_kernels(ws, th + a.w2, a.c2 * a.c1);
   stage_wait();
@@ -639,7 +643,7 @@ __device__ __forceinline__ void rebuild_dz2(float* dst, const ConvArgs& a, int g
 }
 
 // Gradient with respect to conv1's pooled outputs through the ReLU mask, before its routing
-// through pool1: a block per kBackPer28 samples, a thread per sample, input channel and pair of
+// through pool1: a block per back_per samples, a thread per sample, input channel and pair of
 // rows (py0, py0 + 1): the kernel's 25 weights and each row of dz2 are read once for both.
 // The rows y of dz2 come from py0 + 1 down, so that each output row adds its kernel rows
 // from 0 up.  The threads of a warp share the pair (samples and channels vary: 30 of 32 lanes
@@ -649,17 +653,17 @@ constexpr int kBackThreads28 = 192;
 __global__ void __launch_bounds__(kBackThreads28) conv2_back28_kernel(const __grid_constant__ ConvArgs a) {
   gem::pdl_entry();
   extern __shared__ __align__(16) float sm[];
-  const int per_g = (a.b + kBackPer28 - 1) / kBackPer28;
-  const int g = blockIdx.x / per_g, i0 = (blockIdx.x - g * per_g) * kBackPer28;
-  const int ns = min(kBackPer28, a.b - i0);
+  const int per = a.back_per, per_g = (a.b + per - 1) / per;
+  const int g = blockIdx.x / per_g, i0 = (blockIdx.x - g * per_g) * per;
+  const int ns = min(per, a.b - i0);
   const float* th = a.snap + (long long)a.workers[g] * a.snap_stride;
   const int n_dz2 = a.c2 * kH2 * kH2;
   float* ws = sm;                                   // [c2][c1][28]
-  float* dzs = ws + a.c2 * a.c1 * kWPitch;          // [kBackPer28][c2][8][8]
+  float* dzs = ws + a.c2 * a.c1 * kWPitch;          // [back_per][c2][8][8]
   stage_kernels(ws, th + a.w2, a.c2 * a.c1);
   for (int si = 0; si < ns; ++si) rebuild_dz2(dzs + si * n_dz2, a, g, i0 + si);
   stage_wait();
-  const int per_pair = (kBackPer28 * a.c1 + 31) / 32 * 32;   // whole warps
+  const int per_pair = (per * a.c1 + 31) / 32 * 32;   // whole warps
   for (int q = threadIdx.x; q < per_pair * (kP1 / 2); q += blockDim.x) {
     const int pair = q / per_pair, sc = q - pair * per_pair;
     const int si = sc / a.c1, ci = sc - si * a.c1, py0 = 2 * pair;
@@ -926,10 +930,13 @@ int cnn_chunk(gem_cnn* N, const int32_t* workers, int G, const int32_t* rows_dev
   const long long n_pool2 = G * b * s.c2 * s.P2 * s.P2;
   int rc;
   const unsigned samples = unsigned(G * b);
-  const unsigned sample_groups = unsigned(G) * unsigned((b + kPer28 - 1) / kPer28);
+  const bool few = samples <= unsigned(h->sm_count);
+  a.pool2_per = few ? 1 : kPer28;
+  a.back_per = few ? 1 : kBackPer28;
+  auto blocks28 = [&](int per) { return unsigned(G) * unsigned((b + per - 1) / per); };
   if (N->sizes28) {
     gem::launch_pdl(conv1_pool28_kernel, samples, kPool1Threads28, N->smem[0], st, a);
-    gem::launch_pdl(conv2_pool28_kernel, sample_groups, kPool2Threads28, N->smem[1], st, a);
+    gem::launch_pdl(conv2_pool28_kernel, blocks28(a.pool2_per), kPool2Threads28, N->smem[1], st, a);
   } else {
     gem::launch_pdl(s.H == kH ? conv1_pool_kernel<kH> : conv1_pool_kernel<0>, samples, kThreads, N->smem[0], st, a);
     gem::launch_pdl(s.H == kH ? conv2_pool_kernel<kP1> : conv2_pool_kernel<0>, samples, kPool2Threads, N->smem[1], st, a);
@@ -939,8 +946,7 @@ int cnn_chunk(gem_cnn* N, const int32_t* workers, int G, const int32_t* rows_dev
   // the dense head: forward, loss, backward, and the feature gradient
   if ((rc = gem::mlp::mlp_chunk(N->head, workers, G, rows_dev, grads, grad_stride, losses))) return rc;
   if (N->sizes28) {
-    gem::launch_pdl(conv2_back28_kernel, unsigned(G) * unsigned((b + kBackPer28 - 1) / kBackPer28), kBackThreads28,
-                    N->smem[2], st, a);
+    gem::launch_pdl(conv2_back28_kernel, blocks28(a.back_per), kBackThreads28, N->smem[2], st, a);
     gem::launch_pdl(conv2_wpart28_kernel, samples, kW2Threads28, N->smem[3], st, a);
     gem::launch_pdl(conv1_wpart28_kernel, samples, kW1Threads, N->smem[4], st, a);
   } else {
