@@ -45,8 +45,8 @@ int check_handle(const gem_t* h) {
 }
 
 // Launch the commits [0, K) in order; GEM_ECUDA marks the handle broken.
-int launch_commits(gem_t* h, const int* order, const float* const* grads, int K) {
-  return cuda_status(h, gem::commit_ordered(h, order, grads, K));
+int launch_commits(gem_t* h, const int* order, const float* const* grads, int K, bool on_host = false) {
+  return cuda_status(h, gem::commit_ordered(h, order, grads, K, nullptr, nullptr, nullptr, 0, on_host));
 }
 
 int check_batch(const gem_t* h, const int* order, const float* const* grads, int K) {
@@ -81,7 +81,7 @@ namespace gem {
 
 cudaError_t commit_ordered(gem_ctx* h, const int* order, const float* const* grads, int K,
                            float* const* pi_out, unsigned* pi_counts, const long long* pi_seg,
-                           int pi_nseg) {
+                           int pi_nseg, bool grads_on_host) {
   if (pi_counts && (K > kMaxBatchPerLaunch || K * pi_nseg * 2 > kMaxCountWords || !pi_out))
     return cudaErrorInvalidValue;   // counts are kept by one launch
   BatchArgs a;
@@ -89,6 +89,7 @@ cudaError_t commit_ordered(gem_ctx* h, const int* order, const float* const* gra
   a.pi_seg = pi_seg;
   a.pi_nseg = pi_nseg;
   a.lane_rows = 0;
+  a.grads_on_host = grads_on_host ? 1 : 0;
   a.theta = h->theta;
   a.m = h->m;
   a.s = h->s;
@@ -461,7 +462,7 @@ int gem_commit_batch_host(gem_t* h, const int* order, const float* const* grads,
                  aligned16(attr.devicePointer);
       dev[size_t(k)] = static_cast<const float*>(attr.devicePointer);
     }
-    if (in_place) return launch_commits(h, order, dev.data(), K);
+    if (in_place) return launch_commits(h, order, dev.data(), K, true);
   }
   rc = ensure_staging(h);
   if (rc) return rc;

@@ -90,6 +90,7 @@ struct BatchArgsT {
   const long long* pi_seg;                 // device array [pi_nseg + 1], non-decreasing
   int pi_nseg;
   int lane_rows;                           // dynamic shared memory: rows of a 16-byte lane per thread
+  int grads_on_host;                       // 1: the gradients lie in page-locked host memory
   int grads_through_l1;                    // 1: the copies of the gradients are cached in L1
 };
 using BatchArgs = BatchArgsT<kMaxBatchPerLaunch>;
@@ -157,9 +158,10 @@ namespace gem {
 // must have been checked.
 // With pi_counts set (K * pi_nseg * 2 <= kMaxCountWords, one launch), the recording launch
 // also adds the factor counts of every commit and segment to pi_counts (see BatchArgsT).
+// grads_on_host: the gradients are read from page-locked host memory.
 cudaError_t commit_ordered(gem_ctx* h, const int* order, const float* const* grads, int K,
                            float* const* pi_out = nullptr, unsigned* pi_counts = nullptr,
-                           const long long* pi_seg = nullptr, int pi_nseg = 0);
+                           const long long* pi_seg = nullptr, int pi_nseg = 0, bool grads_on_host = false);
 
 // Segments per median call and commits per select launch.
 constexpr int kMaxPiSegments = 64;

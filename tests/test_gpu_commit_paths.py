@@ -127,3 +127,28 @@ def test_gradient_rows_at_every_alignment(P, offsets, rule):
         assert torch.equal(A.theta(), B.theta())
         for w in range(3):
             assert torch.equal(A.snapshot(w), B.snapshot(w)) and torch.equal(A.moment(w), B.moment(w))
+
+
+@pytest.mark.parametrize("offset", [0, 4, 28])
+@pytest.mark.parametrize("rule", [0, 1, 5])
+def test_host_gradient_rows_at_every_alignment(offset, rule):
+    """Page-locked gradients on 128-byte lines and between them, read in place: the bits of the
+    same batch from device memory."""
+    P, n, order = 20_003, 3, [0, 1, 2, 0, 0, 1, 2, 2]
+    rng = np.random.default_rng(offset + rule)
+    ld = (P + 31) // 32 * 32 + 32
+    host = torch.from_numpy((0.1 * rng.standard_normal((len(order), ld))).astype(np.float32)).pin_memory()
+    theta0 = torch.from_numpy(rng.standard_normal(P).astype(np.float32)).cuda()
+    dev = host.cuda()
+    assert host.data_ptr() % 128 == 0 and dev.data_ptr() % 128 == 0
+    with gem.Gem(P, n, 0.01, 0.9, 1e-8) as A, gem.Gem(P, n, 0.01, 0.9, 1e-8) as B:
+        for G in (A, B):
+            G.set_theta(theta0)
+            G.set_mode(rule, 1.5)
+        A.commit_batch_host(order, [host[k, offset:offset + P] for k in range(len(order))])
+        B.commit_batch(order, [dev[k, offset:offset + P].clone() for k in range(len(order))])
+        A.sync()
+        B.sync()
+        assert torch.equal(A.theta(), B.theta())
+        for w in range(n):
+            assert torch.equal(A.snapshot(w), B.snapshot(w)) and torch.equal(A.moment(w), B.moment(w))
