@@ -2,7 +2,9 @@
 
 The quotients are compared with numpy's IEEE division bit for bit over every significand of the
 denominator, which is what the refinement of the reciprocal depends on, and over the
-operand ranges on both sides of the kernel's range check.  The batches are compared with single
+operand ranges on both sides of the kernel's range check: with eps = 1e-18, just above its lower
+end, the kernel divides by itself wherever the operands allow it, with 1e-38 by the
+intrinsic everywhere.  The batches are compared with single
 commits, and those with the oracle by test_gpu_commit.
 """
 import numpy as np
@@ -39,25 +41,31 @@ def _factors(g, m, s, eta, mu, eps):
     return got, want
 
 
+@pytest.mark.parametrize("eps", [1e-18, 1e-38])
 @pytest.mark.parametrize("exponents", [(-1, 1), (-30, 30), (-70, 70), (-126, 126)])
-def test_factor_quotients_are_correctly_rounded(exponents):
-    """Every significand of the denominator (eta = 1, eps negligible: den = |g|), numerators
+def test_factor_quotients_are_correctly_rounded(exponents, eps):
+    """Every significand of the denominator (eta = 1 and, for |g| >= 2^-30, den = |g|), numerators
     and exponents at random; (-70, 70) and (-126, 126) reach past the range check."""
     lo, hi = exponents
     rng = np.random.default_rng(hi)
     P = 1 << 23
     den = np.ldexp((np.arange(P, dtype=np.float64) + P) / P, rng.integers(lo, hi, P)).astype(np.float32)
     num = np.ldexp(1 + rng.random(P), rng.integers(lo, hi, P)).astype(np.float32)
-    got, want = _factors(den, num, np.zeros(P, np.float32), 1.0, 0.9375, 1e-38)
+    got, want = _factors(den, num, np.zeros(P, np.float32), 1.0, 0.9375, eps)
     assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
 
 
-def test_factor_quotients_of_the_largest_significand():
-    """den = 2 - 2^-23, the one denominator whose refined reciprocal may miss round to nearest."""
+@pytest.mark.parametrize("eps", [1e-18, 1e-38])
+@pytest.mark.parametrize("exponent", [-25, 0, 25])
+def test_factor_quotients_of_the_largest_significand(exponent, eps):
+    """den = 2 - 2^-23 times a power of two, the one denominator whose refined reciprocal may miss
+    round to nearest; a numerator that is a power of two then shows it."""
     P = 1 << 23
-    den = np.full(P, 2.0 - 2.0 ** -23, np.float32)
-    num = ((np.arange(P, dtype=np.float64) + P) / P * 8).astype(np.float32)
-    got, want = _factors(den, num, np.zeros(P, np.float32), 1.0, 0.9375, 1e-38)
+    den = np.full(P, np.ldexp(2.0 - 2.0 ** -23, exponent), np.float32)
+    m = np.ldexp((np.arange(P, dtype=np.float64) + P) / P * 8, exponent).astype(np.float32)
+    energy = np.abs(np.float32(0.9375) * m - den)
+    assert (np.frexp(energy)[0] == 0.5).any()
+    got, want = _factors(den, m, np.zeros(P, np.float32), 1.0, 0.9375, eps)
     assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
 
 
