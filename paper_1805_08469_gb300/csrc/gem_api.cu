@@ -94,7 +94,6 @@ cudaError_t commit_ordered(gem_ctx* h, const int* order, const float* const* gra
   a.m = h->m;
   a.s = h->s;
   a.P = h->P;
-  a.stride = h->stride;
   a.eta = h->eta;
   a.mu = h->mu;
   a.eps = h->eps;

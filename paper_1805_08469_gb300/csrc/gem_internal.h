@@ -12,7 +12,7 @@
 namespace gem {
 
 // Commits carried by one launch of the batched commit kernel.  They travel in the
-// kernel's parameter block (2.4 KB + header), so a launch needs no device-side
+// kernel's parameter block (6.4 KB and a header), so a launch needs no device-side
 // descriptor; longer batches are split into several launches, in order.
 constexpr int kMaxBatchPerLaunch = 200;
 
@@ -75,7 +75,6 @@ struct BatchArgsT {
   float* m;                                // [n][stride]
   float* s;                                // [n][stride]
   size_t P;
-  size_t stride;
   float eta, mu, eps;
   int K;                                   // commits in this launch, 1..KCAP
   int rule;                                // RuleKind

@@ -1429,17 +1429,7 @@ int simt_split(int M, int N, int K, int groups, bool can_split) {
 template <int BM, bool AK, bool BK_, int EPI, bool TF32>
 cudaError_t launch_simt_tile(const GemmArgs& a, int groups, cudaStream_t st) {
   constexpr int bytes = 4 * simt_smem_floats(BM, AK, BK_);
-  if (bytes > 40 * 1024) {   // with the row indices beyond the default limit
-    static bool configured[64] = {};   // one attribute call per instantiation and device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !configured[dev]) {
-      const cudaError_t e = cudaFuncSetAttribute(gemm_simt_kernel<BM, AK, BK_, EPI, TF32>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) configured[dev] = true;
-    }
-  }
+  static_assert(bytes <= 40 * 1024, "with the row indices within the default limit");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned((a.N + BN - 1) / BN), unsigned((a.M + BM - 1) / BM), unsigned(groups * a.ksplit));
   cfg.blockDim = dim3(kSimtThreads);
@@ -1788,8 +1778,8 @@ int mlp_chunk(gem_mlp* M, const int32_t* workers, int G, const int32_t* batch_ro
     ba.first[l + 1] = ba.first[l] + M->dims[l + 1];
   }
   // Small networks: the weight and bias gradients in one launch, once the deltas are known; on
-  // the main stream, or on the side stream next to the input gradient and what the caller
-  // does with it.
+  // the main stream, or on the side stream next to the input gradient's product, which the
+  // main stream joins below.
   bool merged = !tf32;
   for (int l = 0; l < L; ++l) merged = merged && small_product(M->dims[l + 1], M->dims[l], b, G);
   const bool aside = merged && two_streams && M->input_grad;

@@ -6,9 +6,12 @@
 //   - every kernel launched with launch_pdl() calls pdl_entry() before it touches global
 //     memory: griddepcontrol.wait returns once the previous grid in the stream has completed
 //     and its writes are visible;
-//   - no kernel triggers its dependents early, so the next launch is scheduled when this
-//     grid's blocks have exited: an earlier trigger let the dependents' blocks crowd onto
-//     the SMs that freed first and made the per-sample kernels slower;
+//   - the next launch is scheduled when this grid's blocks have exited, because no kernel
+//     triggers its dependents before that, but one: an earlier trigger let the dependents'
+//     blocks crowd onto the SMs that freed first and made the per-sample kernels slower.  The
+//     single commit (commit_one_kernel) triggers when it starts, so the kernel after it may be
+//     running before the commit, or what precedes the commit, has ended.  So no kernel may
+//     touch global memory before its wait, whatever it follows;
 //   - dependencies that are not on a kernel of the same stream (event waits, copies) stay
 //     full dependencies.
 // In a kernel launched without the attribute, the wait returns at once.

@@ -133,3 +133,34 @@ def test_minibatch_rows_of_every_entry_point(dims, precision, b, rows):
                                  want_losses=True)
     assert rel_l2(theta, th) < (2e-3 if tf32 else 1e-4)
     np.testing.assert_allclose(run_losses.cpu().numpy(), ref, rtol=2e-3 if tf32 else 1e-4)
+
+
+@pytest.mark.parametrize("dims,G", [([100, 72, 40, 10], 3), ([100, 1000, 516, 10], 2)])
+@pytest.mark.parametrize("layout", ["rows", "spaced"])
+def test_tf32_gradients_are_the_same_wherever_the_caller_wants_them(dims, G, layout):
+    """The tensor cores' weight gradients in the caller's rows directly: the bits of the same call
+    with rows in reverse order, which are copied, and nothing outside the P floats of a row."""
+    b, seed = 48, 5
+    P = synth.mlp_param_count(dims)
+    ld = (P + 3) // 4 * 4 + (64 if layout == "spaced" else 0)
+    X = torch.empty((300, dims[0]), device="cuda")
+    y = torch.empty(300, dtype=torch.int32, device="cuda")
+    synth_gpu.data(seed, X, y, 10)
+    rows = np.random.default_rng(1).integers(0, 300, (G, b)).astype(np.int32)
+    at = list(range(1, G + 1))
+    direct = torch.full((G + 2, ld), -7.0, device="cuda")
+    copied = torch.full((G + 2, ld), -7.0, device="cuda")
+    with gem.Gem(P, G, 0.01, 0.9, 1e-8) as Gh:
+        Gh.set_theta(synth_gpu.xavier(seed, dims, torch.empty(P, device="cuda")))
+        M = sim.gem_mlp_create(Gh.h, dims, b, sim.GEM_MLP_TF32)
+        sim.gem_mlp_set_data(M, X, y)
+        sim.gem_mlp_grad(M, list(range(G)), rows, [direct[i, :P] for i in at])
+        sim.gem_mlp_grad(M, list(range(G)), rows, [copied[G + 1 - i, :P] for i in at])
+        sim.gem_mlp_status(M)
+        sim.gem_mlp_destroy(M)
+    for i in at:
+        assert torch.equal(direct[i, :P], copied[G + 1 - i, :P])
+        assert bool((direct[i, :P] != -7.0).all())
+    mask = torch.ones_like(direct, dtype=torch.bool)
+    mask[1:G + 1, :P] = False
+    assert bool((direct[mask] == -7.0).all()) and bool((copied[mask] == -7.0).all())
