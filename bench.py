@@ -52,8 +52,8 @@ FALLBACK_HBM_GBS = 6800.0
 # on the device), scaled by P: the traffic per coordinate does not depend on P (captures at
 # P = 2,500,000 and 5,000,000 agree within 1%).  Valid only for the kernel source it was
 # taken on (NCU_TRAFFIC_SOURCE_SHA, a hash of the kernel's sources); null once that changes.
-NCU_TRAFFIC_BYTES_PER_LAUNCH = 5 * (7_422_885_632 + 7_097_584_640) // 2   # mean of two launches at P = 5M
-NCU_TRAFFIC_SOURCE_SHA = "865f1023c6c530fb"
+NCU_TRAFFIC_BYTES_PER_LAUNCH = 5 * (7_422_722_816 + 7_099_161_344) // 2   # mean of two launches at P = 5M
+NCU_TRAFFIC_SOURCE_SHA = "6025a0b836834d83"
 NCU_TRAFFIC_HOW = "two launches captured at P=5,000,000 (n=100, K=100), scaled by P to 25,000,000"
 
 
@@ -425,7 +425,7 @@ def run_gem(args, world, rank, local, pg):
             gbs_single = 28 * P_FULL / (ms_single * 1e-3) / 1e9
             single = {"commits_per_s": round(1e3 / ms_single, 1), "ms_per_commit": round(ms_single, 5),
                       "GB_per_s": round(gbs_single, 1), "commits": n_single,
-                      "bytes_per_param": 28, "kernel": "commit_batch_kernel (one commit per launch)",
+                      "bytes_per_param": 28, "kernel": "commit_one_kernel",
                       "note": "gem_commit calls back to back at P=25M, n=100; each launch waits on "
                               "its predecessor, so ms_per_commit bounds the kernel time from above"}
 
